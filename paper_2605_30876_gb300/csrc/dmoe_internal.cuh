@@ -92,17 +92,24 @@ struct Workspace {
   int n_max;           // token tile (MMA N) of the expert GEMMs
 };
 
-// Token tile (MMA N) of the general expert kernel: every group's rows are covered by tiles
-// of n_max rows (a tile of at most half of that loads a half-height box). Each tile streams
-// the group's weights through its SM again, so the tile is as wide as the forward allows:
-// 128 rows, or 256 in block mode with blocks of 16 or more tokens at 1024 or more tokens
-// (every unique expert then takes whole blocks, hundreds of rows; one K box per stage keeps
-// four stages in shared memory).
+// Token tile (MMA N, at most 256) of the general expert kernel: every group's rows are covered
+// by tiles of n_max rows, half of them in each CTA of a pair. Each tile streams the group's
+// weights through its SMs again, so the tile is as wide as the forward allows.
+//
+// Block routing: tiles of whole blocks, where the blocks allow it. A half tile is whole 16-row
+// steps (N is a multiple of 32) and whole blocks, each a box of its own that starts on a 1 KB
+// swizzle boundary (8 rows): the tile is a multiple of 2 blk (blk % 16 = 0) or 4 blk (blk %
+// 16 = 8). 0: no such tile of at most 256 rows.
+inline int expert_tile_unit(int blk) {
+  const int unit = blk % 16 == 0 ? 2 * blk : (blk % 8 == 0 ? 4 * blk : 0);
+  return unit <= 256 ? unit : 0;
+}
 inline int expert_n_max(const dmoe_layer_desc& d) {
   const int T = d.n_blocks * d.block_size;
-  const int cap = (d.mode == DMOE_ROUTE_BLOCK && d.block_size >= 16 && T >= 1024) ? 256 : 128;
-  int n = ((T + 15) / 16) * 16;
-  return n > cap ? cap : (n < 16 ? 16 : n);
+  const bool block = d.mode == DMOE_ROUTE_BLOCK;
+  const int unit = block && expert_tile_unit(d.block_size) > 0 ? expert_tile_unit(d.block_size) : 32;
+  const int n = (T + unit - 1) / unit * unit;
+  return n > 256 ? 256 / unit * unit : n;
 }
 
 Workspace plan_workspace(const dmoe_layer_desc& d);

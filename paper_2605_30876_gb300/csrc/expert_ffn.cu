@@ -1,31 +1,39 @@
 // Expert execution of the MoE layer: grouped SwiGLU FFN over the unique experts of one
 // forward (plus the shared expert), on tcgen05 tensor cores.
 //
-// Both GEMMs are "swap-AB": the expert weights are the MMA's M operand (128 weight rows per
-// tile, streamed by TMA with the 128-byte swizzle), the few tokens routed to an expert are
-// the N operand, K is the reduction dimension, and the fp32 accumulator lives in TMEM.
+// Both GEMMs are "swap-AB": the expert weights are the MMA's M operand (streamed by TMA with
+// the 128-byte swizzle), the tokens routed to an expert are the N operand, K is the reduction
+// dimension, and the fp32 accumulator lives in TMEM. Two CTAs on neighbouring SMs (a cluster
+// of two) share every MMA (cta_group::2, M = 256): each brings its own 128 weight rows and
+// half of the token rows, so that a 128 x 256 x 64 step of one SM takes 32 KB from L2 instead
+// of 48 KB. What one SM can pull from L2 bounds this launch once an expert has many tokens.
 //
 //   gather_kernel       x rows in dispatch order -> xperm [T*k, d]; clears the tile counters
 //   moe_experts_kernel  one persistent launch with two kinds of unit:
-//     gate/up unit      (group, 64 rows of I, token tile): the A tile stacks 64 rows of
-//                       W_gate over the same 64 rows of W_up, so one M=128 MMA chain gives
-//                       gate (TMEM lanes 0-63) and up (lanes 64-127) of those rows; the
-//                       epilogue warps holding "up" pass it through shared memory to the
-//                       warps holding "gate", which write h = silu(gate) * up as bf16 H and
-//                       then publish the tile (h_ready counter)
-//     down unit         (group, 128 rows of d, token tile): D = W_down * H^T; the epilogue
+//     gate/up unit      (group, 128 rows of I, token tile): each CTA's A tile holds 64 rows of
+//                       W_gate and the same 64 rows of W_up, 16 rows of each in turn, so one
+//                       MMA chain leaves gate and up of a row in one warp's TMEM lanes (l and
+//                       l + 16); the two lanes swap half of their columns by shuffles, write
+//                       h = silu(gate) * up as bf16 H and then publish the tile (h_ready
+//                       counter)
+//     down unit         (group, 256 rows of d, token tile): D = W_down * H^T; the epilogue
 //                       stores the rows per (token, slot) as bf16 (half the bytes of fp32
 //                       through HBM twice; the combine adds them in fp32)
 //   combine_kernel      y_t = sum over slots (slot order) of g_tj * row + shared -> bf16
 //
 // A group is one unique expert (dispatch order) or the shared expert (all T tokens). The
-// expert kernel is warp-specialised: warp 0 issues TMA, warp 1 issues MMAs, warps 2-9 run
-// the epilogue; each pipeline stage carries K = 128 (two 128-B-wide boxes per operand; 64
-// for 256-row token tiles). The unit list is derived on
+// expert kernel is warp-specialised: warp 0 issues the TMA loads of the weights, warp 10 those
+// of the token rows, warp 1 of the cluster's first CTA the MMAs, warp 11 hands out the units
+// and watches for their token rows, warps 2-9 run the epilogue. The unit list is derived on
 // the device from the dispatch output, so no host round-trip is needed. Consecutive
 // kernels are chained with programmatic dependent launch: each kernel's set-up (barriers,
 // TMEM, tensor-map prefetch) overlaps the previous kernel, and griddepcontrol.wait orders
 // the reads of its outputs.
+//
+// What bounds it, measured (d = 2048, I = 512, E = 256, k = 8, bias 0.5): at 2048 tokens with
+// block top-k the gate/up units run at 1.8 PFLOP/s while the MMAs alone, with no loads at
+// all, run at 1.85 (a 256 x 256 x 16 pair MMA every 86 ns; cuBLAS peaks at 1.92); with token
+// routing the gate/up phase streams weights at 6.5 TB/s (a copy: 6.7).
 #include <math.h>
 
 #include <mutex>
@@ -37,16 +45,21 @@
 namespace dmoe {
 namespace {
 
-constexpr int kThreads = 320;                      // 10 warps
+constexpr int kThreads = 384;                      // 12 warps
 constexpr int kEpiThreads = 256;                   // warps 2-9: the epilogue
-constexpr int kBoxBytes = 64 * 128;                // one TMA box: 64 rows x 128 B
-constexpr int kMaxKBoxes = 2;                      // K boxes per stage: 1 or 2 (K = 64, 128)
-constexpr int kATileBytes = kTileM * 128;          // 16 KB: 128 rows x 64 K (one K box)
+constexpr int kRowWarp = 10;                       // the producer of the token rows
+constexpr int kPlanWarp = 11;                      // decodes the units, watches for their H tiles
+constexpr int kCluster = 2;                        // CTAs that share an MMA
+constexpr int kGateRows = 16;                      // rows of W_gate, then of W_up, in an A tile
+constexpr int kATileBytes = kTileM * 128;          // 16 KB: 128 rows x 64 K
+constexpr int kLevels = 3;                         // heights of the token row boxes
 constexpr int kMaxGroups = kMaxExperts + 1;
 constexpr uint64_t kWaitTimeoutNs = 1000000000ull;  // 1 s
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 12;                     // ring slots of the weights, at most
+constexpr int kRowStages = 4;                      // ring slots of the token rows
+constexpr int kProgress = 64;                      // steps (K = 128) whose completion is remembered
 constexpr int64_t kDownPrefetchMax = (int64_t)64 << 20;   // half of the 129 MB L2
-constexpr int kXchgStride = 17;                    // floats per row of the exchange buffers
+constexpr int kQueue = 4;                          // units handed out and not yet taken up by every role
 constexpr int kSpecBlocks = 64;                    // blocks of a block top-k forward, at most
 constexpr int kSpecPairs = kSpecBlocks * kMaxTopK;   // (block, coreset member) pairs, at most
 
@@ -60,46 +73,48 @@ struct GemmParams {
   __nv_bfloat16* yslot;   // [T*k, d] bf16 (the combine sums them in fp32)
   __nv_bfloat16* yshared; // [T, d] bf16
   int32_t* h_ready;       // [(E+1) * ntiles]: gate/up tiles done per (group, token tile)
+  int32_t* next_unit;     // units handed out beyond every cluster's first
   DevErrRecord* err;
   const void* w_down;     // routed W_down, prefetched into L2 for the unique experts
   const void* ws_gate; const void* ws_up; const void* ws_down;  // shared, prefetched if set
   int T, d, E, k, I, Is;
-  int n_max;              // token tile = rows of the B box
-  int n_half;             // rows of the half box (token tiles of at most this many rows)
-  int kbs;                // K boxes per stage (1 for 256-row token tiles, else 2)
-  int dpair;              // 128-row tiles of W_down per down unit (2: a pair sharing the H
-                          // stages, K = 64 per stage; 1)
+  int n_max;              // token tile, at most; a multiple of
+  int unit;               // rows that every tile is a multiple of (expert_tile_unit(blk) or 32)
+  int box[kLevels];       // rows of the token row boxes: n_max / 2 (a CTA's half), and smaller
   int ntiles;             // token tiles per group at most
-  int stages;
+  int a_stages, b_stages; // ring slots: 128 weight rows x K = 64, and box[0] x K = 64 of token rows
+                          // (a shorter box leaves room for more of K in a slot)
   int n_acc;              // accumulator buffers in TMEM
+  uint32_t acc_cols;      // ... columns apart
   uint32_t tmem_cols;
   int has_shared;
+  int gu_box, sgu_box;    // gate and up rows come in one box (Maps::gu / sgu): 1: gate first,
+                          // 2: up first; 0: a box per 16 rows (routed experts, shared expert)
   // Block top-k (spec_words != nullptr): the groups come from the coresets that the block
   // routing launch publishes (n_blocks blocks of blk rows). The unique experts are their
   // union, ascending; an expert's token rows are its blocks' rows in block order, which is
-  // the dispatch's order. This launch then does the dispatch itself: its CTAs copy every
-  // (block, coreset member) pair's rows of x to their place in xperm (x_ready[g ntiles + n]
-  // counts the copied rows of token tile n of group g; a gate/up unit loads its tile's rows
-  // once they are all there) and write
-  // n_unique, unique_ids and pos (the row of every (token, slot), from topk_idx).
+  // the dispatch's order. Each token tile is whole blocks, read from x block by block (a box
+  // of blk rows each), so the rows are not copied into dispatch order first; and this launch
+  // writes the dispatch's outputs n_unique, unique_ids and pos (the row of every (token,
+  // slot), from topk_idx).
   const uint32_t* spec_words;
   int n_blocks, blk;
   const int32_t* topk_idx;
   int32_t* pos_out;
   int32_t* n_unique_out;
   int32_t* unique_ids_out;
-  int32_t* x_ready;          // [groups x ntiles], zero at the start (the routing launch
-                             // clears it)
-  const __nv_bfloat16* x;
-  __nv_bfloat16* xperm;
 };
 
+// Weights and the shared expert's rows: [rows, K] in boxes of 64 columns (K). Routed token rows:
+// [rows, K] seen as [K / 64][rows][64], so that one box brings several K steps of few rows.
 struct Maps {
-  CUtensorMap wg, wu, sg, su;   // gate/up weights, 64-row boxes (routed [E*I,d], shared [Is,d])
+  CUtensorMap wg, wu, sg, su;   // gate/up weights, 16-row boxes (routed [E*I,d], shared [Is,d])
+  CUtensorMap gu, sgu;          // both at once: [rows / 16][2][16][d], 64 rows of each in one box
   CUtensorMap wd, sd;           // down weights, 128-row boxes (routed [E*d,I], shared [d,Is])
-  CUtensorMap xp, x;            // gate/up token rows: xperm [T*k,d], x [T,d]
-  CUtensorMap h, hs;            // down token rows: H [T*k,I], Hs [T,Is]
-  CUtensorMap xph, hh;          // xperm and H with half-height boxes (small token tiles)
+  CUtensorMap x, hs;            // shared expert's token rows: x [T,d], Hs [T,Is]
+  CUtensorMap xp[kLevels];      // gate/up token rows xperm [T*k,d] by box height
+  CUtensorMap h[kLevels];       // down token rows H [T*k,I] by box height
+  CUtensorMap xb;               // block top-k: x in boxes of one block
 };
 
 using ptx::fence_proxy_async_global;
@@ -107,14 +122,35 @@ using ptx::ld_acquire;
 using ptx::named_bar_sync;
 using ptx::red_release_add;
 
-__device__ __forceinline__ float silu_f(float z) { return z / (1.f + __expf(-z)); }
+// silu with the fast divide: H is rounded to bf16 right after
+__device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __expf(-z)); }
 
-// A bf16 store that asks L2 to keep the line (the slot rows are read back by the combine
-// right after this launch, while the weights stream through L2 with evict-first)
-__device__ __forceinline__ void st_bf16_keep(__nv_bfloat16* p, __nv_bfloat16 v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.b16 [%0], %1, %2;" ::"l"(p),
-               "h"(*reinterpret_cast<const unsigned short*>(&v)), "l"(pol)
-               : "memory");
+// A store that asks L2 to keep the line (the slot rows are read back by the combine right
+// after this launch, while the weights stream through L2 with evict-first)
+__device__ __forceinline__ void st_u32_keep(void* p, uint32_t v, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
+}
+
+// A thread holds eight tokens' values of one row; the row of lane xor 1 is its neighbour. After
+// the swap it holds two neighbouring rows (the lower one first) of four tokens: the even
+// lane tokens 0-3, the odd lane tokens 4-7, one bf16 pair per token, so that a warp's stores
+// are 4-byte words of 64-byte runs (half the stores of single bf16 values).
+__device__ __forceinline__ void pair_rows(const float (&v)[8], uint32_t (&w)[4]) {
+  uint32_t pk[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    pk[i] = *reinterpret_cast<const uint32_t*>(&b);
+  }
+  const bool odd = threadIdx.x & 1;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t mine = odd ? pk[2 + i] : pk[i];
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, odd ? pk[i] : pk[2 + i], 1);
+    const uint32_t lo = odd ? other : mine, hi = odd ? mine : other;
+    w[2 * i] = __byte_perm(lo, hi, 0x5410);
+    w[2 * i + 1] = __byte_perm(lo, hi, 0x7632);
+  }
 }
 
 // AND of `v` over the kEpiThreads epilogue threads (named barrier 1), so that they take the
@@ -133,11 +169,14 @@ __device__ __forceinline__ bool epi_all_threads(bool v) {
 }
 
 // Debug builds (-DDMOE_TRACE) record a per-CTA timeline of the expert kernel: slot 0 entry,
-// 1 after the unit list, 62 exit; for the i-th unit of the CTA (i < 8), at 2 + 6i: unit id,
-// producer start, last TMA issued, H ready (down units; for block top-k gate/up units: the
-// group's token rows copied), last MMA commit, epilogue done;
-// at 50 + i: the epilogue's first TMEM read of that unit; 63: this CTA's copies of the
-// token rows done (block top-k).
+// 1 after the unit list, 62 exit; for the i-th unit of the CTA from
+// DMOE_TRACE_UNIT0 on (i < 8), at 2 + 6i: unit id,
+// weight producer start, last weight load issued, H ready (down units), last MMA commit,
+// epilogue done; at 50 + i: the epilogue's first TMEM read of that unit.
+#ifndef DMOE_TRACE_UNIT0
+#define DMOE_TRACE_UNIT0 0   // the first unit of a CTA that is recorded
+#endif
+#define TRU(i) ((unsigned)((i) - DMOE_TRACE_UNIT0))
 #ifdef DMOE_TRACE
 __device__ uint64_t g_trace[kMaxPersistentCtas * 64];
 #define DMOE_TRACE_AT(slot) (g_trace[blockIdx.x * 64 + (slot)] = ptx::globaltimer_ns())
@@ -148,12 +187,15 @@ __device__ uint64_t g_trace[kMaxPersistentCtas * 64];
 #endif
 
 // The expert FFN of one forward in one persistent launch. Units: first every gate/up tile
-// (group, 64 rows of I, token tile), then every down tile (group, 128 rows of d, token
-// tile); the shared expert's group comes first in both lists. A CTA takes units
-// blockIdx.x, blockIdx.x + gridDim.x, ... so its gate/up units always precede its down
-// units and a gate/up unit never waits on another unit. A down unit loads its W_down
-// tiles at once and only then waits (bounded) for the gate/up tiles of its token rows to
-// be published (h_ready), so weight streaming of both phases overlaps. kSpec: the block
+// (group, 128 rows of I, token tile), then every down tile (group, 256 rows of d, token
+// tile); the shared expert's group comes first in both lists. A cluster's first unit is its
+// number; it takes every further one from a global counter when it begins to load the one
+// before (units differ in cost, and a fixed share left the last cluster 12-20 us behind the
+// first at 256 to 2048 tokens). A
+// cluster's unit numbers ascend, so its gate/up units precede its down units and a gate/up
+// unit never waits on another unit. The weights of a down unit are loaded as ring slots free;
+// only its token rows wait (bounded) for the gate/up tiles of those rows to be published
+// (h_ready), so weight streaming of both phases overlaps. kSpec: the block
 // top-k form (GemmParams::spec_words), compiled separately so that the other form carries
 // none of its code.
 template <bool kSpec>
@@ -163,26 +205,29 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   const uint32_t raw_addr = ptx::smem_addr(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);  // 1024-B aligned
 
-  const int stages = p.stages;
-  const int kbs = p.kbs;                                      // K boxes per stage
-  const int stage_k = kbs * kTileK;
-  const uint32_t a_stage = (uint32_t)kbs * kATileBytes;
-  const uint32_t b_box = (uint32_t)p.n_max * 128u;            // one B box (slot size)
-  const uint32_t b_stage = (uint32_t)kbs * b_box;
+  const int a_stages = p.a_stages, b_stages = p.b_stages;
+  const uint32_t b_slot = (uint32_t)p.box[0] * 128u;
   const uint32_t off_a = 0;
-  const uint32_t off_b = off_a + (uint32_t)stages * a_stage;
-  const uint32_t off_x = off_b + (uint32_t)stages * b_stage;
-  const uint32_t x_bytes = 2u * 128u * kXchgStride * 4u;       // 2 x [128][17] fp32
-  const uint32_t off_bar = (off_x + x_bytes + 7u) & ~7u;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + off_bar);
-  uint64_t* empty = full + stages;
-  uint64_t* acc_full = empty + stages;
+  const uint32_t off_b = off_a + (uint32_t)a_stages * kATileBytes;
+  const uint32_t off_bar = off_b + (uint32_t)b_stages * b_slot;
+  uint64_t* a_full = reinterpret_cast<uint64_t*>(smem + off_bar);
+  uint64_t* b_full = a_full + a_stages;
+  uint64_t* progress = b_full + b_stages;          // step t done: phase t / kProgress of entry
+                                                   // t % kProgress
+  uint64_t* acc_full = progress + kProgress;
   uint64_t* acc_empty = acc_full + 4;
   uint64_t* drain = acc_empty + 4;
-  int* misc = reinterpret_cast<int*>(drain + 1);
+  uint64_t* q_full = drain + 1;                    // the queue of units: entry i written
+  uint64_t* q_empty = q_full + kQueue;             // ... and read by both CTAs (first CTA's)
+  uint64_t* d_full = q_empty + kQueue;             // the same units decoded: entry written
+  uint64_t* d_empty = d_full + kQueue;             // ... and read by every role of the CTA
+  int2* s_desc = reinterpret_cast<int2*>(d_empty + kQueue);   // [kQueue]
+  int* misc = reinterpret_cast<int*>(s_desc + kQueue);
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(misc + 0);
   volatile int* s_abort = misc + 1;
-  int* s_sched = misc + 4;                         // G, U, gu_units, dn_units, dpair
+  int* s_rows_ok = misc + 2;                       // units whose token rows are there
+  volatile int* s_queue = misc + 8;                // [kQueue]
+  int* s_sched = misc + 4;                         // G, U, gu_units, dn_units
   int* gu_prefix = misc + 12;                      // [kMaxGroups + 1], by slot
   int* dn_prefix = gu_prefix + (kMaxGroups + 1);   // [kMaxGroups + 1], by slot
   int* g_row0 = dn_prefix + (kMaxGroups + 1);      // by group
@@ -194,36 +239,60 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   int16_t* s_upos = reinterpret_cast<int16_t*>(s_bmask + 2 * kMaxExperts);   // [kMaxExperts]
   int16_t* s_bpos = s_upos + kMaxExperts;                                      // [kMaxExperts]
   uint8_t* s_bcore = reinterpret_cast<uint8_t*>(s_bpos + kMaxExperts);   // [kSpecPairs]
-  float* xchg = reinterpret_cast<float*>(smem + off_x);
 
+  constexpr bool spec = kSpec;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)ptx::cluster_ctarank();
+  const int cl = (int)blockIdx.x / kCluster, ncl = (int)gridDim.x / kCluster;
   if (tid == 0) DMOE_TRACE_AT(0);
   KLOG(DMOE_KERNEL_EXPERTS, 0);
 
   if (tid == 0) {
-    for (int s = 0; s < stages; ++s) {
-      ptx::mbar_init(&full[s], 1);
-      ptx::mbar_init(&empty[s], 1);
-    }
+    for (int s = 0; s < a_stages; ++s) ptx::mbar_init(&a_full[s], 1);
+    for (int s = 0; s < b_stages; ++s) ptx::mbar_init(&b_full[s], 1);
+    for (int s = 0; s < kProgress; ++s) ptx::mbar_init(&progress[s], 1);
     for (int a = 0; a < 4; ++a) {
       ptx::mbar_init(&acc_full[a], 1);
-      ptx::mbar_init(&acc_empty[a], kEpiThreads);
+      ptx::mbar_init(&acc_empty[a], kCluster * kEpiThreads / 32);   // every epilogue warp
     }
     ptx::mbar_init(drain, 1);
+    for (int i = 0; i < kQueue; ++i) {
+      ptx::mbar_init(&q_full[i], 1);
+      ptx::mbar_init(&q_empty[i], kCluster);
+      ptx::mbar_init(&d_full[i], 1);
+      // the two producers, the epilogue warps and, in the first CTA, the MMA issuer
+      ptx::mbar_init(&d_empty[i], 2 + kEpiThreads / 32 + (rank == 0 ? 1 : 0));
+      ptx::mbar_arrive_expect_tx(&q_full[i], 4);   // the entry's first unit
+    }
+    *s_rows_ok = 0;
     ptx::fence_mbarrier_init();
     *s_abort = 0;
-    ptx::prefetch_tensormap(&tm.wg);
-    ptx::prefetch_tensormap(&tm.wu);
+    ptx::prefetch_tensormap(&tm.gu);
     ptx::prefetch_tensormap(&tm.wd);
-    ptx::prefetch_tensormap(&tm.xp);
-    ptx::prefetch_tensormap(&tm.h);
+    ptx::prefetch_tensormap(spec ? &tm.xb : &tm.xp[0]);
+    ptx::prefetch_tensormap(&tm.h[0]);
   }
   if (warp == 1) {
-    ptx::tmem_alloc(s_tmem, p.tmem_cols);
-    ptx::tmem_relinquish();
+    ptx::tmem_alloc2(s_tmem, p.tmem_cols);
+    ptx::tmem_relinquish2();
   }
-  constexpr bool spec = kSpec;
-  if (!spec) pdl_wait();  // dispatch output and the gathered rows are complete from here on
+  ptx::cluster_arrive();   // the barriers of both CTAs are set up
+  ptx::cluster_wait();
+  // No dependency wait here. The launch before this one (the dispatch placement or the gather)
+  // released it after its own wait, so the unique list and the offsets are complete; what that
+  // launch itself writes (the rows in dispatch order, the zeroed counters) is used by the row
+  // producer, the plan warp's polls and the unit counter, which wait first. The weights of the
+  // first unit are on their way by then.
+
+  // Enters the cluster's unit i >= 1 into the queue of both CTAs (one thread of the first CTA;
+  // the entry's last unit must have been read by both).
+  auto enter_unit = [&](int i, int u) {
+    const int e = (i - 1) % kQueue;
+#pragma unroll
+    for (int r = 0; r < kCluster; ++r)
+      ptx::st_async_u32(ptx::peer_smem(const_cast<const int*>(s_queue) + e, r), (uint32_t)u,
+                        ptx::peer_smem(&q_full[e], r));
+  };
 
   // ---------------- groups and unit lists (slot 0 = the shared expert when present)
   if (warp == 0) {
@@ -347,8 +416,8 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         g_cnt[g] = cnt;
         g_e[g] = e;
         const int nt = (cnt + p.n_max - 1) / p.n_max;
-        gu = nt * (Ig / 64);
-        dn = nt * (p.d / kTileM);
+        gu = nt * (Ig / 128);
+        dn = nt * ((p.d + 255) / 256);
       }
       int igu = gu, idn = dn;
 #pragma unroll
@@ -364,15 +433,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       carry_gu += __shfl_sync(0xffffffffu, igu, 31);
       carry_dn += __shfl_sync(0xffffffffu, idn, 31);
     }
-    // pairs of down tiles only when the down units are many per CTA (a pair unit pulls 25 %
-    // less per tile but holds less of its weights before H is ready: with about one or two
-    // single units per CTA it lengthens the tail); a pair count is the single count / 2
-    const int dpair = (p.dpair == 2 && carry_dn >= 4 * (int)gridDim.x) ? 2 : 1;
-    if (dpair == 2) {
-      __syncwarp();
-      for (int i = lane; i <= G; i += 32) dn_prefix[i] /= 2;
-      carry_dn /= 2;
-    }
     if (lane == 0) {
       gu_prefix[0] = 0;
       dn_prefix[0] = 0;
@@ -380,7 +440,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       s_sched[1] = U;
       s_sched[2] = carry_gu;
       s_sched[3] = carry_dn;
-      s_sched[4] = dpair;
     }
   }
   ptx::tc_fence_before();
@@ -388,7 +447,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   ptx::tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   const int G = s_sched[0], U = s_sched[1], n_gu = s_sched[2], n_dn = s_sched[3];
-  const int dpair = s_sched[4];   // 128-row tiles of W_down per down unit
   const int units = n_gu + n_dn;
   if (tid == 0) DMOE_TRACE_AT(1);
   if (tid == 64) {
@@ -416,32 +474,72 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     }
   }
 
-  // unit -> phase, group, m tile, n tile
-  struct Unit { bool gu; int g, m, n; };
-  auto decode = [&](int u) -> Unit {
-    Unit r;
-    r.gu = u < n_gu;
-    const int* pre = r.gu ? gu_prefix : dn_prefix;
-    const int v = r.gu ? u : u - n_gu;
+  // A unit: phase, group, m tile, n tile, rows of the token tile. The plan warp finds it from
+  // its number and passes it on packed in two words (a search and a division of about 0.7 us
+  // per unit, which the tensor pipe would wait for in the issuing thread).
+  struct Unit {
+    bool end, gu, shared;
+    int g, m, n, rows, col0;   // col0: the tile's first row within the group
+  };
+  auto find_unit = [&](int u) -> int2 {
+    if (u >= units) return make_int2(-1, 0);
+    const bool gu = u < n_gu;
+    const int* pre = gu ? gu_prefix : dn_prefix;
+    const int v = gu ? u : u - n_gu;
     int lo = 0, hi = G - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (pre[mid] <= v) lo = mid; else hi = mid - 1;
     }
-    r.g = p.has_shared ? (lo == 0 ? U : lo - 1) : lo;
-    // token tile innermost: the CTAs that take a weight tile's token tiles take them at
+    const int g = p.has_shared ? (lo == 0 ? U : lo - 1) : lo;
+    if (g_cnt[g] <= p.n_max)   // one token tile
+      return make_int2((gu ? 1 : 0) | (g >= U ? 2 : 0) | g_cnt[g] << 2 | (v - pre[lo]) << 12, g);
+    // token tile innermost: the clusters that take a weight tile's token tiles take them at
     // the same time, so that the tile comes from HBM once and from L2 for the others
-    const int nt = (g_cnt[r.g] + p.n_max - 1) / p.n_max;
-    const int local = v - pre[lo];
-    r.m = local / nt;
-    r.n = local - r.m * nt;
+    const int nt = (g_cnt[g] + p.n_max - 1) / p.n_max;
+    const int local = v - pre[lo], m = local / nt, n = local - m * nt;
+    // the group's tiles are of one size (300 rows: 160 + 140, not 256 + 44)
+    const int step = nt * p.unit, tile = (g_cnt[g] + step - 1) / step * p.unit;
+    const int rows = min(tile, g_cnt[g] - n * tile);
+    return make_int2((gu ? 1 : 0) | (g >= U ? 2 : 0) | rows << 2 | m << 12 | n << 20,
+                     g | (n * tile) << 16);
+  };
+  auto unpack = [&](int2 d) -> Unit {
+    Unit r;
+    r.end = d.x < 0;
+    r.gu = d.x & 1;
+    r.shared = d.x & 2;
+    r.rows = (d.x >> 2) & 0x3ff;
+    r.m = (d.x >> 12) & 0xff;
+    r.n = (d.x >> 20) & 0x3f;
+    r.g = d.y & 0xffff;
+    r.col0 = d.y >> 16;
     return r;
   };
-  auto wait = [&](uint64_t* bar, uint32_t parity, int value) -> bool {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+  // token rows per CTA of a unit's MMA (N is twice that, a multiple of 32): half of the tile's
+  // rows, in whole blocks where the rows come from x block by block
+  auto half_of = [&](const Unit& un) -> int {
+    if (spec && un.gu && !un.shared) return (un.rows + p.unit - 1) / p.unit * (p.unit / 2);
+    return (un.rows + 31) / 32 * 16;
+  };
+  // rows of one K step in a slot of token rows: whole blocks, or the smallest box that holds
+  // the half; the slot holds box[0] / rows K steps
+  auto slot_rows = [&](const Unit& un, int half, int* level) -> int {
+    *level = 0;
+    if (un.shared) return p.box[0];
+    if (spec && un.gu) return half;
+    int lv = 0;
+#pragma unroll
+    for (int l = 1; l < kLevels; ++l)
+      if (p.box[l] >= half) lv = l;
+    *level = lv;
+    return lv == 0 ? p.box[0] : (lv == 1 ? p.box[1] : p.box[2]);
+  };
+  auto wait_on = [&](auto try_wait, int value) -> bool {
+    if (try_wait()) return true;
     const uint64_t t0 = ptx::globaltimer_ns();
     for (uint32_t i = 1;; ++i) {
-      if (ptx::mbar_try_wait(bar, parity)) return true;
+      if (try_wait()) return true;
       if ((i & 63u) == 0u) {
         if (*s_abort) return false;
         if (ptx::globaltimer_ns() - t0 > kWaitTimeoutNs) {
@@ -452,305 +550,296 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       }
     }
   };
+  auto wait = [&](uint64_t* bar, uint32_t parity, int value) -> bool {
+    return wait_on([&] { return ptx::mbar_try_wait(bar, parity); }, value);
+  };
+
+  // The cluster's i-th unit for a role of this CTA: a thread, or (warp_wide) a warp, all lanes
+  // of which read it. The entry is free again once all roles have read it.
+  auto unit_at = [&](int i, bool warp_wide) -> Unit {
+    const int e = i % kQueue;
+    const bool got = wait(&d_full[e], (uint32_t)(i / kQueue) & 1u, i);
+    const Unit un = unpack(got ? s_desc[e] : make_int2(-1, 0));
+    if (warp_wide) __syncwarp();
+    if (!warp_wide || lane == 0) ptx::mbar_arrive(&d_empty[e]);
+    return un;
+  };
+  // Steps (K = 128) are counted over all units of the cluster; one commit per step reports to
+  // both CTAs that its MMAs are done, and with them the slots that they read: a commit costs
+  // the issuing thread about 0.1 us, as much as two MMAs. A producer is never kProgress steps
+  // behind a step it waits for (the MMAs run on what it has loaded), so the parity is that of
+  // step t or of no later one.
+  auto step_done = [&](int t, int value) -> bool {
+    return wait(&progress[t % kProgress], (uint32_t)(t / kProgress) & 1u, value);
+  };
+  // after a failed wait: lets this producer's copies in flight land before the CTA exits (they
+  // complete on the first CTA's barriers, together with the other CTA's: a slot that one left
+  // unfilled runs the bounded wait out)
+  auto drain_copies = [&](uint64_t* full, int stages, int st, uint32_t ph, int issued) {
+    for (int i = issued < stages ? issued : stages; i > 0; --i) {
+      if (--st < 0) { st = stages - 1; ph ^= 1u; }
+      const uint64_t t0 = ptx::globaltimer_ns();
+      while ((rank != 0 || !ptx::mbar_try_wait(&full[st], ph)) &&
+             ptx::globaltimer_ns() - t0 < kWaitTimeoutNs / 10) {
+      }
+    }
+  };
 
   if (warp == 0) {
-    // ================= TMA producer
+    // ================= TMA producer of the weights: waits for ring slots only, so the weights
+    // of the next unit follow those of the last without a gap. The bytes of both CTAs
+    // complete on the first CTA's barriers, where its producers expect them.
     if (lane == 0) {
       const uint64_t pol_first = ptx::policy_evict_first();   // weights read by one tile
       const uint64_t pol_norm = ptx::policy_evict_normal();   // ... or by several
-      const uint64_t pol_x = ptx::policy_evict_last();    // activations: re-read by tiles
-      int stage = 0;
+      const uint32_t full0 = ptx::peer_smem(a_full, 0);
+      int stage = 0, chunk = 0;
       uint32_t phase = 0;
-      int issued = 0;
       bool ok = true;
-      int li = 0;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++li) {
-        const Unit un = decode(u);
-        const bool shared = un.g >= U;
+      for (int i = 0; ok; ++i) {
+        const Unit un = unit_at(i, false);
+        if (un.end) break;
+        const bool shared = un.shared;
         const uint64_t pol_w = g_cnt[un.g] > p.n_max ? pol_norm : pol_first;
-        // a routed token tile of at most n_half rows loads the half-height box
-        const int nvalid = min(p.n_max, g_cnt[un.g] - un.n * p.n_max);
-        const bool half = !shared && nvalid <= p.n_half;
-        const uint32_t b_bytes = (uint32_t)kbs * (half ? (uint32_t)p.n_half * 128u : b_box);
-        const uint32_t tx_bytes = a_stage + b_bytes;
-        if (li < 8) { DMOE_TRACE_SET(2 + 6 * li, u); DMOE_TRACE_AT(3 + 6 * li); }
-        if (un.gu) {
-          const int arow = shared ? un.m * 64 : g_e[un.g] * p.I + un.m * 64;
-          const int brow = (shared ? 0 : g_row0[un.g]) + un.n * p.n_max;
-          const CUtensorMap* mg = shared ? &tm.sg : &tm.wg;
-          const CUtensorMap* mu = shared ? &tm.su : &tm.wu;
-          const CUtensorMap* mb = shared ? &tm.x : (half ? &tm.xph : &tm.xp);
-          const int kc = p.d / stage_k;
-          auto load_gu = [&](int st, int c, bool with_a, bool with_b) {
-            uint8_t* a_dst = smem + off_a + st * a_stage;
-            uint8_t* b_dst = smem + off_b + st * b_stage;
-            for (int kb = 0; kb < kbs; ++kb) {
-              const int kx = c * stage_k + kb * kTileK;
-              if (with_a) {
-                ptx::tma_load_2d(a_dst + kb * kATileBytes, mg, &full[st], kx, arow, pol_w);
-                ptx::tma_load_2d(a_dst + kb * kATileBytes + kBoxBytes, mu, &full[st], kx, arow,
-                                 pol_w);
-              }
-              if (with_b) ptx::tma_load_2d(b_dst + kb * b_box, mb, &full[st], kx, brow, pol_x);
+        if (TRU(i) < 8) { DMOE_TRACE_SET(2 + 6 * TRU(i), un.gu); DMOE_TRACE_AT(3 + 6 * TRU(i)); }
+        // the next unit: the first CTA asks for it now and enters it for both CTAs once half
+        // of this unit's loads are issued
+        int next = units;
+        if (rank == 0 && i > 0) next = ncl + atomicAdd(p.next_unit, 1);
+        const int kc = (un.gu ? p.d : (shared ? p.Is : p.I)) / kTileK;
+        // (d % 256 = 128: the last down unit's second half reads the rows that follow and
+        // stores nothing)
+        const int arow = un.gu ? (shared ? 0 : g_e[un.g] * p.I) + un.m * 128 + rank * 64
+                               : (shared ? 0 : g_e[un.g] * p.d) + un.m * 256 + rank * kTileM;
+        const int one_box = shared ? p.sgu_box : p.gu_box;
+        const CUtensorMap* m0 = un.gu ? (shared ? &tm.sg : &tm.wg) : (shared ? &tm.sd : &tm.wd);
+        const CUtensorMap* m1 = shared ? &tm.su : &tm.wu;
+        const CUtensorMap* m01 = shared ? &tm.sgu : &tm.gu;
+        for (int c = 0; c < kc; ++c, ++chunk) {
+          // the slot's last K step was chunk - a_stages
+          if (chunk >= a_stages && !step_done((chunk - a_stages) >> 1, i)) { ok = false; break; }
+          if (rank == 0) ptx::mbar_arrive_expect_tx(&a_full[stage], kCluster * kATileBytes);
+          uint8_t* dst = smem + off_a + stage * kATileBytes;
+          const uint32_t bar = full0 + 8u * (uint32_t)stage;
+          if (!un.gu) {
+            ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow, pol_w);
+          } else if (one_box != 0) {
+            ptx::tma_load_4d_pair(dst, m01, bar, c * kTileK, 0, 0, arow / kGateRows, pol_w);
+          } else {
+            for (int r = 0; r < 64; r += kGateRows, dst += 2 * kGateRows * 128) {
+              ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow + r, pol_w);
+              ptx::tma_load_2d_pair(dst + kGateRows * 128, m1, bar, c * kTileK, arow + r, pol_w);
             }
-          };
-          int c0 = 0;
-          if (spec && !shared) {
-            // block top-k: the weight stages first, the token rows once this launch's copies
-            // of the tile's rows are all in xperm
-            const int pre = kc < stages ? kc : stages;
-            const int stage0 = stage;
-            for (int c = 0; c < pre; ++c) {
-              if (!wait(&empty[stage], phase ^ 1u, u)) { ok = false; break; }
-              ptx::mbar_arrive_expect_tx(&full[stage], tx_bytes);
-              load_gu(stage, c, true, false);
-              ++issued;
-              if (++stage == stages) { stage = 0; phase ^= 1u; }
-            }
-            if (!ok) break;
-            // the rows of this token tile (a pair's rows lie in one tile: n_max % blk == 0)
-            const int32_t* flag = p.x_ready + un.g * p.ntiles + un.n;
-            const int need = min(p.n_max, g_cnt[un.g] - un.n * p.n_max);
-            if (ld_acquire(flag) < need) {
-              const uint64_t t0 = ptx::globaltimer_ns();
-              while (ld_acquire(flag) < need) {
-                if (*s_abort) { ok = false; break; }
-                if (ptx::globaltimer_ns() - t0 > kWaitTimeoutNs) {
-                  record_error(p.err, kErrTimeout, kAtGather, u);
-                  *s_abort = 1;
-                  ok = false;
-                  break;
-                }
-              }
-            }
-            fence_proxy_async_global();   // the copies (generic stores) before these loads
-            if (li < 8) DMOE_TRACE_AT(5 + 6 * li);
-            int st = stage0;
-            for (int c = 0; c < pre; ++c) {
-              if (ok)
-                load_gu(st, c, false, true);
-              else
-                ptx::mbar_complete_tx_local(&full[st], b_bytes);   // keep the accounting whole
-              if (++st == stages) st = 0;
-            }
-            if (!ok) break;
-            c0 = pre;
           }
-          for (int c = c0; c < kc; ++c) {
-            if (!wait(&empty[stage], phase ^ 1u, u)) { ok = false; break; }
-            ptx::mbar_arrive_expect_tx(&full[stage], tx_bytes);
-            load_gu(stage, c, true, true);
-            ++issued;
-            if (++stage == stages) { stage = 0; phase ^= 1u; }
-          }
-        } else {
-          // a pair unit takes 128-row tiles 2m and 2m+1 of W_down over K = 64 per stage (its
-          // two A boxes side by side at the same K), both against the stage's one H box
-          const bool pr = dpair == 2;
-          const int ksz = pr ? kTileK : stage_k;               // K per stage
-          const int nbb = pr ? 1 : kbs;                        // B boxes per stage
-          const uint32_t b_bytes_d =
-              (uint32_t)nbb * (half ? (uint32_t)p.n_half * 128u : b_box);
-          const uint32_t tx_d = a_stage + b_bytes_d;
-          const int Kg = shared ? p.Is : p.I;
-          const int arow = (shared ? 0 : g_e[un.g] * p.d) + un.m * dpair * kTileM;
-          const int brow = (shared ? 0 : g_row0[un.g]) + un.n * p.n_max;
-          const CUtensorMap* ma = shared ? &tm.sd : &tm.wd;
-          const CUtensorMap* mb = shared ? &tm.hs : (half ? &tm.hh : &tm.h);
-          const int kc = Kg / ksz;
-          const int pre = kc < stages ? kc : stages;
-          const int stage0 = stage;
-          auto load_a = [&](int st, int c) {
-            uint8_t* a_dst = smem + off_a + st * a_stage;
-            if (pr) {
-              ptx::tma_load_2d(a_dst, ma, &full[st], c * ksz, arow, pol_w);
-              ptx::tma_load_2d(a_dst + kATileBytes, ma, &full[st], c * ksz, arow + kTileM, pol_w);
-            } else {
-              for (int kb = 0; kb < kbs; ++kb)
-                ptx::tma_load_2d(a_dst + kb * kATileBytes, ma, &full[st], c * ksz + kb * kTileK,
-                                 arow, pol_w);
+          if (++stage == a_stages) { stage = 0; phase ^= 1u; }
+          if (rank == 0 && c == kc / 2) {
+            if (i == 0) {
+              if (!spec) pdl_wait();   // the counter is zero from here on
+              next = ncl + atomicAdd(p.next_unit, 1);
             }
-          };
-          // weights first: they do not depend on the gate/up phase
-          for (int c = 0; c < pre; ++c) {
-            if (!wait(&empty[stage], phase ^ 1u, u)) { ok = false; break; }
-            ptx::mbar_arrive_expect_tx(&full[stage], tx_d);
-            load_a(stage, c);
-            ++issued;
-            if (++stage == stages) { stage = 0; phase ^= 1u; }
+            if (i >= kQueue && !wait(&q_empty[i % kQueue], ((i / kQueue) & 1) ^ 1, i)) {
+              ok = false;
+              break;
+            }
+            enter_unit(i + 1, next);
           }
+        }
+        if (TRU(i) < 8) DMOE_TRACE_AT(4 + 6 * TRU(i));
+      }
+      if (!ok) drain_copies(a_full, a_stages, stage, phase, chunk);
+    }
+  } else if (warp == kRowWarp) {
+    // ================= TMA producer of the token rows (x or H; lane i issues the i-th box of a
+    // slot): at the start of a down unit it waits until every gate/up tile of its token tile
+    // is published
+    const uint64_t pol_x = ptx::policy_evict_last();    // activations: re-read by tiles
+    const uint32_t full0 = ptx::peer_smem(b_full, 0);
+    int stage = 0, issued = 0;
+    uint32_t phase = 0;
+    int step0 = 0;          // the unit's first step
+    if (!spec) pdl_wait();   // the rows in dispatch order are complete from here on
+    int last = 0;           // lane s: the last step that reads what slot s holds
+    bool ok = true;
+    for (int i = 0; ok; ++i) {
+      const Unit un = unit_at(i, true);
+      if (!__all_sync(0xffffffffu, !un.end)) break;
+      const bool shared = un.shared;
+      const int half = half_of(un);
+      const int Kg = un.gu ? p.d : (shared ? p.Is : p.I);
+      int lv;
+      const int rows = slot_rows(un, half, &lv);    // per K step
+      const int kpb = p.box[0] / rows;              // K steps per slot
+      int nbox = 1;                                 // boxes per K step
+      int y = (shared ? 0 : g_row0[un.g]) + un.col0 + rank * half;
+      const CUtensorMap* mb = un.gu ? (shared ? &tm.x : &tm.xp[lv]) : (shared ? &tm.hs : &tm.h[lv]);
+      if (spec && un.gu && !shared) {
+        // this CTA's blocks of the tile, from the group's blocks in ascending order (past the
+        // last one any block: its columns are not used)
+        nbox = half / p.blk;
+        mb = &tm.xb;
+        const uint32_t* bm = s_bmask + 2 * g_e[un.g];
+        uint64_t m = (uint64_t)bm[0] | ((uint64_t)bm[1] << 32);
+        for (int b = un.col0 / p.blk + rank * nbox + lane % nbox; b > 0 && (m & (m - 1)); --b)
+          m &= m - 1;
+        y = (__ffsll((long long)m) - 1) * p.blk;
+      }
+      if (!un.gu) {
+        // (the plan warp has seen them; its acquire carries over)
+        ok = wait_on(
+            [&] {
+              if (ptx::ld_acquire_cta(s_rows_ok) > i) return true;
+              __nanosleep(32);
+              return false;
+            },
+            i);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        fence_proxy_async_global();   // generic stores of the rows before these loads
+        if (lane == 0 && TRU(i) < 8) DMOE_TRACE_AT(5 + 6 * TRU(i));
+      }
+      const uint32_t box_bytes = (uint32_t)(rows / nbox) * 128u;
+      const int kc = Kg / kTileK;
+      const bool by_block = spec && un.gu && !shared;
+      for (int c = 0; c < kc; c += kpb) {
+        if (issued >= b_stages) {
+          ok = __all_sync(0xffffffffu, step_done(__shfl_sync(0xffffffffu, last, stage), i));
           if (!ok) break;
-          // then the H rows, once every gate/up tile of this token tile is published
-          const int target = Kg / 64;
+        }
+        uint8_t* dst = smem + off_b + stage * b_slot;
+        const uint32_t bar = full0 + 8u * (uint32_t)stage;
+        if (by_block) {
+          const int n = min(kpb, kc - c) * nbox;      // boxes of this slot (at most 16)
+          if (lane == 0 && rank == 0)
+            ptx::mbar_arrive_expect_tx(&b_full[stage], kCluster * (uint32_t)n * box_bytes);
+          if (lane < n)
+            ptx::tma_load_2d_pair(dst + lane * box_bytes, mb, bar, (c + lane / nbox) * kTileK, y,
+                                  pol_x);
+        } else if (lane == 0) {
+          // (kpb K steps in one box; steps past the end of K read as zeros)
+          if (rank == 0)
+            ptx::mbar_arrive_expect_tx(&b_full[stage], kCluster * (uint32_t)kpb * box_bytes);
+          if (shared)
+            ptx::tma_load_2d_pair(dst, mb, bar, c * kTileK, y, pol_x);
+          else
+            ptx::tma_load_3d_pair(dst, mb, bar, 0, y, c, pol_x);
+        }
+        if (lane == stage) last = step0 + (min(c + kpb, kc) - 1) / 2;
+        ++issued;
+        if (++stage == b_stages) { stage = 0; phase ^= 1u; }
+      }
+      step0 += kc / 2;
+    }
+    if (!ok && lane == 0) drain_copies(b_full, b_stages, stage, phase, issued);
+  } else if (warp == kPlanWarp) {
+    // ================= the units, decoded one or more ahead of their use, and the readiness of
+    // their token rows (a poll is an L2 round trip, 1 us or more while weights stream)
+    if (lane == 0) {
+      const uint32_t q_empty0 = ptx::peer_smem(q_empty, 0);
+      for (int i = 0;; ++i) {
+        int u = cl;
+        if (i > 0) {
+          const int q = (i - 1) % kQueue;
+          u = wait(&q_full[q], (uint32_t)((i - 1) / kQueue) & 1u, i) ? s_queue[q] : units;
+          ptx::mbar_arrive_expect_tx(&q_full[q], 4);   // the entry's next unit
+          ptx::mbar_arrive_pair(q_empty0 + 8u * (uint32_t)q);
+        }
+        const int2 d = find_unit(u);
+        const int e = i % kQueue;
+        if (i >= kQueue && !wait(&d_empty[e], ((uint32_t)(i / kQueue) & 1u) ^ 1u, i)) break;
+        s_desc[e] = d;
+        ptx::mbar_arrive(&d_full[e]);
+        const Unit un = unpack(d);
+        if (un.end) break;
+        if (!un.gu) {
+          if (!spec) pdl_wait();   // the counters are zeroed from here on
           const int32_t* flag = p.h_ready + un.g * p.ntiles + un.n;
-          if (ld_acquire(flag) < target) {
+          const int need = (un.shared ? p.Is : p.I) / 64;
+          bool ok = true;
+          if (ld_acquire(flag) < need) {
             const uint64_t t0 = ptx::globaltimer_ns();
-            while (ld_acquire(flag) < target) {
+            while (ok && ld_acquire(flag) < need) {
               __nanosleep(64);
-              if (*s_abort) { ok = false; break; }
+              if (*s_abort) ok = false;
               if (ptx::globaltimer_ns() - t0 > kWaitTimeoutNs) {
                 record_error(p.err, kErrTimeout, kAtDown, u);
                 *s_abort = 1;
-                ok = false;
-                break;
               }
             }
           }
-          fence_proxy_async_global();
-          if (li < 8) DMOE_TRACE_AT(5 + 6 * li);
-          int st = stage0;
-          for (int c = 0; c < pre; ++c) {
-            if (ok) {
-              uint8_t* b_dst = smem + off_b + st * b_stage;
-              for (int kb = 0; kb < nbb; ++kb)
-                ptx::tma_load_2d(b_dst + kb * b_box, mb, &full[st], c * ksz + kb * kTileK, brow,
-                                 pol_x);
-            } else {
-              // keep the barrier accounting whole: complete the stage without B data
-              ptx::mbar_complete_tx_local(&full[st], b_bytes_d);
-            }
-            if (++st == stages) st = 0;
-          }
           if (!ok) break;
-          for (int c = pre; c < kc; ++c) {
-            if (!wait(&empty[stage], phase ^ 1u, u)) { ok = false; break; }
-            ptx::mbar_arrive_expect_tx(&full[stage], tx_d);
-            load_a(stage, c);
-            uint8_t* b_dst = smem + off_b + stage * b_stage;
-            for (int kb = 0; kb < nbb; ++kb)
-              ptx::tma_load_2d(b_dst + kb * b_box, mb, &full[stage], c * ksz + kb * kTileK, brow,
-                               pol_x);
-            ++issued;
-            if (++stage == stages) { stage = 0; phase ^= 1u; }
-          }
         }
-        if (li < 8) DMOE_TRACE_AT(4 + 6 * li);
-      }
-      if (!ok) {
-        // let the copies already in flight land before the CTA exits
-        int st = stage;
-        uint32_t ph = phase;
-        const int n = issued < stages ? issued : stages;
-        for (int i = 0; i < n; ++i) {
-          if (--st < 0) { st = stages - 1; ph ^= 1u; }
-          const uint64_t t0 = ptx::globaltimer_ns();
-          while (!ptx::mbar_try_wait(&full[st], ph) &&
-                 ptx::globaltimer_ns() - t0 < kWaitTimeoutNs / 10) {
-          }
-        }
+        ptx::st_release_cta(s_rows_ok, i + 1);
       }
     }
   } else if (warp == 1) {
-    // ================= MMA issuer
-    if (lane == 0) {
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0;
+    // ================= MMA issuer: the first CTA's, for both. The tensor pipe queues one or two
+    // MMAs, so this thread's pauses are the pipe's: the next slots are tested while MMAs are
+    // queued.
+    if (rank == 0 && lane == 0) {
+      int sa = 0, sb = 0, acc = 0, step = 0;
+      bool a_in = false, b_in = false;      // the next slots were seen full
+      uint32_t pa = 0, pb = 0, acc_phase = 0;
       bool ok = true;
-      int li = 0;
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++li) {
-        const Unit un = decode(u);
-        const bool shared = un.g >= U;
-        const bool pr = !un.gu && dpair == 2;     // a pair of down tiles, two accumulators
-        const int Kg = un.gu ? p.d : (shared ? p.Is : p.I);
-        const int kc = Kg / (pr ? kTileK : stage_k);
-        const int nvalid = min(p.n_max, g_cnt[un.g] - un.n * p.n_max);
-        const uint32_t n_mma = (uint32_t)((nvalid + 15) & ~15);
-        const uint32_t idesc = ptx::idesc_bf16(kTileM, n_mma);
-        // the second accumulator of a pair: the next slot
-        int acc2 = acc + 1;
-        uint32_t acc2_phase = acc_phase;
-        if (acc2 == p.n_acc) { acc2 = 0; acc2_phase ^= 1u; }
-        if (!wait(&acc_empty[acc], acc_phase ^ 1u, u)) { ok = false; break; }
-        if (pr && !wait(&acc_empty[acc2], acc2_phase ^ 1u, u)) { ok = false; break; }
-        ptx::tc_fence_after();
-        const uint32_t d0 = tmem_base + (uint32_t)acc * (uint32_t)p.n_max;
-        const uint32_t d1 = tmem_base + (uint32_t)acc2 * (uint32_t)p.n_max;
-        for (int c = 0; c < kc; ++c) {
-          if (!wait(&full[stage], phase, u)) { ok = false; break; }
+      for (int i = 0; ok; ++i) {
+        const Unit un = unit_at(i, false);
+        if (un.end) break;
+        const int steps = (un.gu ? p.d : (un.shared ? p.Is : p.I)) / (2 * kTileK);
+        const int half = half_of(un);
+        const uint32_t idesc = ptx::idesc_bf16(kCluster * kTileM, (uint32_t)(2 * half));
+        int lv;
+        const uint32_t step_bytes = (uint32_t)slot_rows(un, half, &lv) * 128u;
+        const int kpb = (int)(b_slot / step_bytes);
+        {
+          ok = wait(&acc_empty[acc], acc_phase ^ 1u, i);
           ptx::tc_fence_after();
-          if (!*s_abort) {
-            const uint32_t a0 = ptx::smem_addr(smem + off_a + stage * a_stage);
-            const uint32_t b0 = ptx::smem_addr(smem + off_b + stage * b_stage);
-            if (pr) {
+          const uint32_t d0 = tmem_base + (uint32_t)acc * p.acc_cols;
+          const uint32_t a0 = ptx::smem_addr(smem + off_a), b0 = ptx::smem_addr(smem + off_b);
+          int kb = kpb - 1;           // K box within the slot of token rows
+          uint32_t bs = 0;
+          for (int c = 0; ok && c < steps; ++c, ++step) {
+#pragma unroll
+            for (int k2 = 0; k2 < 2; ++k2) {
+              ok = ok && (a_in || wait(&a_full[sa], pa, i));
+              const uint32_t as = a0 + (uint32_t)sa * kATileBytes;
+              if (++sa == a_stages) { sa = 0; pa ^= 1u; }
+              bs += step_bytes;
+              if (++kb == kpb) {      // the next slot
+                ok = ok && (b_in || wait(&b_full[sb], pb, i));
+                bs = b0 + (uint32_t)sb * b_slot;
+                kb = 0;
+                if (++sb == b_stages) { sb = 0; pb ^= 1u; }
+              }
+              if (!ok) break;
+              ptx::tc_fence_after();
 #pragma unroll
               for (int kk = 0; kk < kTileK / 16; ++kk) {
-                const uint64_t bd = ptx::sdesc_k_sw128(b0 + kk * 32);
-                const uint32_t accum = (c > 0 || kk > 0) ? 1u : 0u;
-                ptx::mma_bf16(d0, ptx::sdesc_k_sw128(a0 + kk * 32), bd, idesc, accum);
-                ptx::mma_bf16(d1, ptx::sdesc_k_sw128(a0 + kATileBytes + kk * 32), bd, idesc,
-                              accum);
+                ptx::mma_bf16_pair(d0, ptx::sdesc_k_sw128(as + kk * 32),
+                                   ptx::sdesc_k_sw128(bs + kk * 32), idesc,
+                                   (c > 0 || k2 > 0 || kk > 0) ? 1u : 0u);
+                if (kk == 1) {
+                  a_in = ptx::mbar_test_wait(&a_full[sa], pa);
+                  b_in = ptx::mbar_test_wait(&b_full[sb], pb);
+                }
               }
-            } else {
-              for (int kb = 0; kb < kbs; ++kb)
-#pragma unroll
-                for (int kk = 0; kk < kTileK / 16; ++kk)
-                  ptx::mma_bf16(d0, ptx::sdesc_k_sw128(a0 + kb * kATileBytes + kk * 32),
-                                ptx::sdesc_k_sw128(b0 + kb * b_box + kk * 32), idesc,
-                                (c > 0 || kb > 0 || kk > 0) ? 1u : 0u);
             }
+            if (!ok) break;
+            ptx::mma_commit_pair(&progress[step % kProgress]);
           }
-          ptx::mma_commit(&empty[stage]);
-          if (++stage == stages) { stage = 0; phase ^= 1u; }
-        }
-        if (!ok) break;
-        ptx::mma_commit(&acc_full[acc]);
-        if (pr) ptx::mma_commit(&acc_full[acc2]);
-        if (li < 8) DMOE_TRACE_AT(6 + 6 * li);
-        if (pr) {
-          acc = acc2;
-          acc_phase = acc2_phase;
+          if (ok) ptx::mma_commit_pair(&acc_full[acc]);
+          if (TRU(i) < 8) DMOE_TRACE_AT(6 + 6 * TRU(i));
         }
         if (++acc == p.n_acc) { acc = 0; acc_phase ^= 1u; }
       }
       // make sure no MMA is still running when TMEM is released
-      ptx::mma_commit(drain);
+      ptx::mma_commit_pair(drain);
       const uint64_t t0 = ptx::globaltimer_ns();
       while (!ptx::mbar_try_wait(drain, 0) && ptx::globaltimer_ns() - t0 < kWaitTimeoutNs) {
       }
     }
   } else {
     // ================= epilogue: warps 2..9, TMEM lanes 32*(warp%4) ..; two column groups
-    // (warps 2-5 and 6-9) take alternate 16-column slices of the accumulator, each with its
-    // own exchange tile and named barrier (the epilogue math is latency-bound: two groups
-    // finish a tile in about half the time)
-    if (spec && U > 0) {
-      // this CTA's share of the dispatch's copies: the rows of pair (block b, coreset member
-      // e) go to xperm rows blk * (s_bpos[e] + rank of b among e's blocks), a pair split into
-      // up to four parts when the pairs are fewer than the CTAs; the group counts its copied
-      // rows (one release add per part, after every epilogue thread's stores)
-      const int et = tid - 64;
-      const int npairs = p.n_blocks * p.k;
-      int parts = (int)gridDim.x / npairs;
-      parts = parts < 1 ? 1 : (parts > 4 ? 4 : parts);
-      while (p.blk % parts != 0) --parts;
-      const int prow = p.blk / parts;                 // rows per part
-      const int n16 = prow * p.d / 8;                 // 16-byte pieces per part
-      for (int w = blockIdx.x; w < npairs * parts; w += gridDim.x) {
-        const int i = w / parts, part = w - i * parts;
-        const int b = i / p.k, e = s_bcore[i];
-        const uint32_t lo = s_bmask[2 * e], hi = s_bmask[2 * e + 1];
-        const int rank = b < 32 ? __popc(lo & ((1u << b) - 1u))
-                                : __popc(lo) + __popc(hi & ((1u << (b - 32)) - 1u));
-        const uint4* src = reinterpret_cast<const uint4*>(
-            p.x + ((size_t)b * p.blk + (size_t)part * prow) * p.d);
-        uint4* dst = reinterpret_cast<uint4*>(
-            p.xperm + ((size_t)p.blk * (s_bpos[e] + rank) + (size_t)part * prow) * p.d);
-        for (int v0 = et; v0 < n16; v0 += kEpiThreads * 8) {
-          uint4 r[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (v0 + q * kEpiThreads < n16) r[q] = __ldg(src + v0 + q * kEpiThreads);
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (v0 + q * kEpiThreads < n16) dst[v0 + q * kEpiThreads] = r[q];
-        }
-        __threadfence();
-        named_bar_sync(4, kEpiThreads);
-        if (et == 0)
-          red_release_add(p.x_ready + s_upos[e] * p.ntiles + (p.blk * rank) / p.n_max, prow);
-      }
-      if (et == 0) DMOE_TRACE_AT(63);
-    }
+    // (warps 2-5 and 6-9) take alternate 16-column slices of the accumulator (the epilogue math
+    // is latency-bound: two groups finish a tile in about half the time)
     if (spec && warp == 2) {
       // the dispatch's outputs: the row of every (token, slot) of this CTA's share of the
       // tokens (expert e = topk_idx[t, j] of block b: the group's rows start at
@@ -787,102 +876,104 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     const int q = warp & 3;
     const int cg = (warp - 2) >> 2;                 // column group
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    float* xg = xchg + cg * (128 * kXchgStride);    // this group's exchange tile
-    const int gbar = 2 + cg;                        // this group's named barrier
+    const int odd = lane & 1;
     const uint64_t pol_keep = ptx::policy_evict_last();   // the slot rows, for the combine
-    int acc = 0, li = 0;
+    const uint32_t acc_empty0 = ptx::peer_smem(acc_empty, 0);
+    int acc = 0;
     uint32_t acc_phase = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x, ++li) {
-      const Unit un = decode(u);
-      const bool shared = un.g >= U;
-      const int nvalid = min(p.n_max, g_cnt[un.g] - un.n * p.n_max);
-      const int n_mma = (nvalid + 15) & ~15;
-      const bool pr = !un.gu && dpair == 2;     // a pair of down tiles: two accumulators
-      int acc2 = acc + 1;
-      uint32_t acc2_phase = acc_phase;
-      if (acc2 == p.n_acc) { acc2 = 0; acc2_phase ^= 1u; }
-      if (!epi_all_threads(wait(&acc_full[acc], acc_phase, u) &&
-                           (!pr || wait(&acc_full[acc2], acc2_phase, u))))
-        break;
+    for (int i = 0;; ++i) {
+      const Unit un = unit_at(i, true);
+      const bool shared = un.shared;
+      const int nvalid = un.rows;
+      // (a warp whose wait failed leaves with the others)
+      if (!epi_all_threads(!un.end && wait(&acc_full[acc], acc_phase, i))) break;
       ptx::tc_fence_after();
-      if (tid == 64 && li < 8) DMOE_TRACE_AT(50 + li);
-      const uint32_t tbase = tmem_base + lane_off + (uint32_t)acc * (uint32_t)p.n_max;
-      const int col0 = un.n * p.n_max;              // first token column of the tile
+      if (tid == 64 && TRU(i) < 8) DMOE_TRACE_AT(50 + TRU(i));
+      const uint32_t tbase = tmem_base + lane_off + (uint32_t)acc * p.acc_cols;
+      const int col0 = un.col0;                     // first token column of the tile
       if (un.gu) {
-        // lanes 0-63: gate rows, lanes 64-127: up rows of the same 64 intermediate units
-        const bool is_gate = q < 2;
-        const int r64 = (q & 1) * 32 + lane;         // row within the 64-row slice
+        // lanes 0-15 of a quadrant: gate rows, lanes 16-31: up rows of the same 16 intermediate
+        // units (or the other way round). Per 16-token slice a gate lane gives its last 8
+        // columns to the lane that holds its row's up values and takes that one's first 8: each
+        // then has gate and up of one row for 8 tokens. Two slices at a time (32 columns apart):
+        // their latencies overlap
         const int Ig = shared ? p.Is : p.I;
-        __nv_bfloat16* hout = shared ? p.hs : p.h;
-        const int hrow0 = (shared ? 0 : g_row0[un.g]) + col0;
-        // per 16-token slice: every accumulator row's 16 values go to the exchange tile
-        // (gate rows 0-63, up rows 64-127), then each of the group's 128 threads takes 8
-        // adjacent H columns of one token (loads, SwiGLU, one 16-byte store). Interleaving
-        // the exchange loads with the H stores instead serialises them: the compiler
-        // cannot tell the two memories apart.
-        const int et = tid - 64 - 128 * cg, xc = et >> 3, hc = (et & 7) * 8;
-        for (int c0 = 16 * cg; c0 < n_mma; c0 += 32) {
-          float v[16];
-          ptx::tmem_ld16(tbase + c0, v);
+        const int row = un.m * 128 + rank * 64 + q * kGateRows + (lane & 15);
+        __nv_bfloat16* hout = (shared ? p.hs : p.h) +
+                              (size_t)((shared ? 0 : g_row0[un.g]) + col0) * Ig + (row & ~1);
+        const bool is_gate = (lane < 16) == ((shared ? p.sgu_box : p.gu_box) != 2);
+        for (int c0 = 16 * cg; c0 < nvalid; c0 += 64) {
+          // (past the last slice the first one again, and nothing is stored)
+          const int c1 = c0 + 32 < nvalid ? c0 + 32 : c0;
+          float v[2][16];
+          ptx::tmem_ld16(tbase + c0, v[0]);
+          ptx::tmem_ld16(tbase + c1, v[1]);
           ptx::tmem_ld_wait();
-          {
-            float* xr = xg + ((is_gate ? 0 : 64) + r64) * kXchgStride;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) xr[c] = v[c];
-          }
-          named_bar_sync(gbar, 128);
-          float gv[8], uv[8];
+          for (int s = 0; s < 2; ++s)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            gv[j] = xg[(hc + j) * kXchgStride + xc];
-            uv[j] = xg[(64 + hc + j) * kXchgStride + xc];
-          }
-          uint32_t hp[4];
+            for (int j = 0; j < 16; ++j) asm volatile("" : "+f"(v[s][j]));   // only after the wait
+          float h[2][8];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(silu_f(gv[2 * j]) * uv[2 * j],
-                                                            silu_f(gv[2 * j + 1]) * uv[2 * j + 1]);
-            hp[j] = *reinterpret_cast<const uint32_t*>(&h2);
+          for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float other =
+                  __shfl_xor_sync(0xffffffffu, is_gate ? v[s][8 + j] : v[s][j], kGateRows);
+              h[s][j] = silu_f(is_gate ? v[s][j] : other) * (is_gate ? other : v[s][8 + j]);
+            }
+#pragma unroll
+          for (int s = 0; s < 2; ++s) {
+            uint32_t w[4];
+            pair_rows(h[s], w);
+            const int t0 = (s == 0 ? c0 : c0 + 32) + (is_gate ? 0 : 8) + 4 * odd;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (t0 + j < nvalid)
+                *reinterpret_cast<uint32_t*>(hout + (size_t)(t0 + j) * Ig) = w[j];
           }
-          if (c0 + xc < nvalid)
-            *reinterpret_cast<uint4*>(hout + (size_t)(hrow0 + c0 + xc) * Ig + un.m * 64 + hc) =
-                make_uint4(hp[0], hp[1], hp[2], hp[3]);
-          named_bar_sync(gbar, 128);   // the exchange tile is rewritten by the next slice
         }
-        if (tid == 64 && li < 4) DMOE_TRACE_AT(54 + li);
         ptx::tc_fence_before();
-        ptx::mbar_arrive(&acc_empty[acc]);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive_pair(acc_empty0 + 8u * (uint32_t)acc);
         // publish the tile: the barrier orders every epilogue thread's H stores before one
         // release add; a reader acquires the counter, then fences the async proxy
         named_bar_sync(4, kEpiThreads);
-        if (tid == 64 && li < 8) DMOE_TRACE_AT(58 + (li < 4 ? li : 3));
         if (tid == 64) red_release_add(p.h_ready + un.g * p.ntiles + un.n, 1);
       } else {
-        __nv_bfloat16* out = shared ? p.yshared + (size_t)col0 * p.d
-                                    : p.yslot + (size_t)(g_row0[un.g] + col0) * p.d;
-        for (int h = 0; h < (pr ? 2 : 1); ++h) {
-          const int slot = h == 0 ? acc : acc2;
-          const uint32_t tb = tmem_base + lane_off + (uint32_t)slot * (uint32_t)p.n_max;
-          const int drow = (un.m * dpair + h) * kTileM + q * 32 + lane;
-          for (int c0 = 16 * cg; c0 < n_mma; c0 += 32) {
-            float v[16];
-            ptx::tmem_ld16(tb + c0, v);
+        const int drow = un.m * 256 + rank * kTileM + q * 32 + lane;
+        __nv_bfloat16* out = (shared ? p.yshared + (size_t)col0 * p.d
+                                     : p.yslot + (size_t)(g_row0[un.g] + col0) * p.d) + (drow & ~1);
+        if (drow < p.d) {   // the same for the whole CTA (d is a multiple of 128)
+          for (int c0 = 16 * cg; c0 < nvalid; c0 += 64) {
+            const int c1 = c0 + 32 < nvalid ? c0 + 32 : c0;
+            float v[2][16];
+            ptx::tmem_ld16(tbase + c0, v[0]);
+            ptx::tmem_ld16(tbase + c1, v[1]);
             ptx::tmem_ld_wait();
 #pragma unroll
-            for (int c = 0; c < 16; ++c)
-              if (c0 + c < nvalid)
-                st_bf16_keep(out + (size_t)(c0 + c) * p.d + drow, __float2bfloat16_rn(v[c]),
-                             pol_keep);
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+              for (int j = 0; j < 16; ++j) asm volatile("" : "+f"(v[s][j]));
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              float h[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) h[j] = v[g >> 1][8 * (g & 1) + j];
+              uint32_t w[4];
+              pair_rows(h, w);
+              const int t0 = c0 + 32 * (g >> 1) + 8 * (g & 1) + 4 * odd;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (t0 + j < nvalid) st_u32_keep(out + (size_t)(t0 + j) * p.d, w[j], pol_keep);
+            }
           }
-          ptx::tc_fence_before();
-          ptx::mbar_arrive(&acc_empty[slot]);
         }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive_pair(acc_empty0 + 8u * (uint32_t)acc);
       }
-      if (tid == 64 && li < 8) DMOE_TRACE_AT(7 + 6 * li);
-      if (pr) {
-        acc = acc2;
-        acc_phase = acc2_phase;
-      }
+      if (tid == 64 && TRU(i) < 8) DMOE_TRACE_AT(7 + 6 * TRU(i));
       if (++acc == p.n_acc) { acc = 0; acc_phase ^= 1u; }
     }
   }
@@ -890,14 +981,18 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
-  // the combine may start now: launched earlier, its waiting CTAs would share the SMs with
-  // this launch and slow it down
+  // the combine may start now (launched earlier, its waiting CTAs would share the SMs with this
+  // launch and slow it down); it reads the placement's output before its own wait
+  pdl_wait();
   pdl_launch_dependents();
   if (tid == 0) DMOE_TRACE_AT(62);
   KLOG(DMOE_KERNEL_EXPERTS, 1);
+  // neither CTA leaves while the other may still signal its barriers or read its tiles
+  ptx::cluster_arrive();
+  ptx::cluster_wait();
   if (warp == 1) {
     __syncwarp();
-    ptx::tmem_dealloc(tmem_base, p.tmem_cols);
+    ptx::tmem_dealloc2(tmem_base, p.tmem_cols);
   }
 }
 
@@ -1058,6 +1153,41 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, ui
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same matrix as [cols / 64][rows][64]: a box of `ksteps` 64-column steps of box_rows rows.
+bool make_map_k(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
+                uint32_t ksteps) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)kTileK, rows, cols / kTileK};
+  const cuuint64_t strides[2] = {cols * 2, (cuuint64_t)kTileK * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)kTileK, box_rows, ksteps};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Two matrices [rows, cols] of one shape as [rows / 16][2][16][cols], the one at the lower
+// address first: one box brings 64 rows of both, 16 of each in turn (a copy costs the SM's copy
+// engine about 100 cycles besides its rows). Their distance is a stride of the map: a multiple
+// of 16 bytes below 2^40. Returns 1 (a first), 2 (b first) or 0: the distance is no such stride,
+// no map is made.
+int make_map_two(CUtensorMap* m, const void* a, const void* b, uint64_t rows, uint64_t cols) {
+  EncodeTiledFn enc = encode_fn();
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  const uint64_t dist = pa < pb ? pb - pa : pa - pb;
+  if (enc == nullptr || dist == 0 || dist % 16 != 0 || dist >= ((uint64_t)1 << 40)) return 0;
+  const cuuint64_t dims[4] = {cols, kGateRows, 2, rows / kGateRows};
+  const cuuint64_t strides[3] = {cols * 2, dist, cols * 2 * kGateRows};
+  const cuuint32_t box[4] = {(cuuint32_t)kTileK, kGateRows, 2, 64 / kGateRows};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  if (enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(pa < pb ? a : b), dims, strides,
+          box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return 0;
+  return pa < pb ? 1 : 2;
+}
+
 uint32_t pow2_cols(uint32_t c) {
   uint32_t r = 32;
   while (r < c) r <<= 1;
@@ -1065,10 +1195,9 @@ uint32_t pow2_cols(uint32_t c) {
 }
 
 size_t experts_fixed_smem() {
-  // alignment slack + exchange buffers + barriers + misc/group arrays + block top-k planning
-  return 1024 + 2 * 128 * kXchgStride * 4 + 8 + 8 * (2 * kMaxStages + 9) +
-         sizeof(int) * (12 + 5 * (kMaxGroups + 1)) + 64 + 4 * 2 * kMaxExperts +
-         2 * 2 * kMaxExperts + kSpecPairs;
+  // alignment slack + barriers + misc/group arrays + block top-k planning
+  return 1024 + 8 * (kMaxStages + kRowStages + kProgress + 9 + 5 * kQueue) + sizeof(int) * (12 + 5 * (kMaxGroups + 1)) +
+         64 + 4 * 2 * kMaxExperts + 2 * 2 * kMaxExperts + kSpecPairs;
 }
 
 int max_smem_optin() {
@@ -1093,15 +1222,15 @@ DMOE_KLOG_EXPORT(dmoe_debug_klog_experts)
 #endif
 
 int experts_ready_counters(int T, int E, int n_max) {
-  return (E + 1) * ((T + n_max - 1) / n_max);
+  return (E + 1) * ((T + n_max - 1) / n_max) + 1;   // and the counter of units
 }
 
 bool experts_spec_ok(const dmoe_layer_desc& d, int n_max) {
-  // blocks of whole 8-row groups (a block's box starts on a 1 KB swizzle boundary), whole
-  // blocks per token tile, at most kSpecBlocks blocks (a 64-bit block mask per expert)
+  // blocks that fill a CTA's half of a token tile whole (expert_tile_unit), at most kSpecBlocks
+  // of them (a 64-bit block mask per expert)
   return d.mode == DMOE_ROUTE_BLOCK && d.top_p <= 0.f && mask_top_k(d) == d.top_k &&
-         d.n_blocks >= 1 && d.n_blocks <= kSpecBlocks && d.block_size % 8 == 0 &&
-         n_max % d.block_size == 0 && d.n_experts <= kMaxExperts;
+         d.n_blocks >= 1 && d.n_blocks <= kSpecBlocks && expert_tile_unit(d.block_size) > 0 &&
+         n_max % expert_tile_unit(d.block_size) == 0 && d.n_experts <= kMaxExperts;
 }
 
 cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
@@ -1129,6 +1258,7 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   gp.yslot = static_cast<__nv_bfloat16*>(a.yslot);
   gp.yshared = static_cast<__nv_bfloat16*>(a.yshared);
   gp.h_ready = a.h_ready;
+  gp.next_unit = a.h_ready + n_ready - 1;
   gp.err = a.err;
   gp.w_down = a.w_down;
   if (has_shared && a.prefetch_shared) {
@@ -1138,56 +1268,63 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   }
   gp.T = a.T; gp.d = a.d; gp.E = a.E; gp.k = a.k; gp.I = a.I; gp.Is = a.Is;
   gp.n_max = a.n_max;
-  gp.n_half = ((a.n_max / 2) + 15) & ~15;
-  gp.kbs = a.n_max >= 256 ? 1 : kMaxKBoxes;
-  // pairs of down tiles share their H stages: 25 % less to pull per SM and half the down
-  // units, so that each CTA takes about one (needs two K boxes per stage for the pair's A
-  // and an even number of 128-row tiles of d)
-  gp.dpair = (gp.kbs == 2 && (a.d / kTileM) % 2 == 0) ? 2 : 1;
+  gp.unit = 32;
+  gp.box[0] = a.n_max / 2;
+  for (int i = 1; i < kLevels; ++i) gp.box[i] = ((gp.box[i - 1] / 2) + 7) & ~7;
   gp.ntiles = (a.T + a.n_max - 1) / a.n_max;
   gp.has_shared = has_shared ? 1 : 0;
   if (spec) {
     gp.spec_words = a.spec_words;
     gp.n_blocks = a.spec_blocks;
     gp.blk = a.T / a.spec_blocks;
+    gp.unit = expert_tile_unit(gp.blk);   // whole blocks
     gp.topk_idx = a.topk_idx;
     gp.pos_out = a.pos_out;
     gp.n_unique_out = a.n_unique_out;
     gp.unique_ids_out = a.unique_ids_out;
-    gp.x_ready = a.h_ready + experts_ready_counters(a.T, a.E, a.n_max);
-    gp.x = a.x;
-    gp.xperm = a.xperm;
   }
 
   // 2. gate/up + SwiGLU and down projection in one persistent launch
-  Maps m;
-  bool ok = make_map(&m.wg, a.w_gate, (uint64_t)a.E * a.I, a.d, 64) &&
-            make_map(&m.wu, a.w_up, (uint64_t)a.E * a.I, a.d, 64) &&
-            make_map(&m.wd, a.w_down, (uint64_t)a.E * a.d, a.I, kTileM) &&
-            make_map(&m.xp, a.xperm, (uint64_t)pairs, a.d, (uint32_t)a.n_max) &&
-            make_map(&m.x, a.x, (uint64_t)a.T, a.d, (uint32_t)a.n_max) &&
-            make_map(&m.h, a.h, (uint64_t)pairs, a.I, (uint32_t)a.n_max) &&
-            make_map(&m.xph, a.xperm, (uint64_t)pairs, a.d, (uint32_t)gp.n_half) &&
-            make_map(&m.hh, a.h, (uint64_t)pairs, a.I, (uint32_t)gp.n_half);
-  if (ok && has_shared)
-    ok = make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, 64) &&
-         make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, 64) &&
-         make_map(&m.sd, a.ws_down, (uint64_t)a.d, a.Is, kTileM) &&
-         make_map(&m.hs, a.hs, (uint64_t)a.T, a.Is, (uint32_t)a.n_max);
-  if (!has_shared) { m.sg = m.wg; m.su = m.wu; m.sd = m.wd; m.hs = m.h; }
+  // (only the maps that this call uses: each costs the host time)
+  Maps m{};
+  const uint64_t gu_rows = (uint64_t)a.E * a.I;
+  bool ok = make_map(&m.wd, a.w_down, (uint64_t)a.E * a.d, a.I, kTileM);
+  gp.gu_box = make_map_two(&m.gu, a.w_gate, a.w_up, gu_rows, a.d);
+  if (gp.gu_box == 0)
+    ok = ok && make_map(&m.wg, a.w_gate, gu_rows, a.d, kGateRows) &&
+         make_map(&m.wu, a.w_up, gu_rows, a.d, kGateRows);
+  if (spec) ok = ok && make_map(&m.xb, a.x, (uint64_t)a.T, a.d, (uint32_t)gp.blk);
+  for (int i = 0; i < kLevels; ++i) {
+    const uint32_t rows = (uint32_t)gp.box[i], ksteps = (uint32_t)(gp.box[0] / gp.box[i]);
+    if (!spec) ok = ok && make_map_k(&m.xp[i], a.xperm, (uint64_t)pairs, a.d, rows, ksteps);
+    ok = ok && make_map_k(&m.h[i], a.h, (uint64_t)pairs, a.I, rows, ksteps);
+  }
+  if (has_shared) {
+    ok = ok && make_map(&m.sd, a.ws_down, (uint64_t)a.d, a.Is, kTileM) &&
+         make_map(&m.x, a.x, (uint64_t)a.T, a.d, (uint32_t)gp.box[0]) &&
+         make_map(&m.hs, a.hs, (uint64_t)a.T, a.Is, (uint32_t)gp.box[0]);
+    gp.sgu_box = make_map_two(&m.sgu, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d);
+    if (gp.sgu_box == 0)
+      ok = ok && make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, kGateRows) &&
+           make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, kGateRows);
+  }
   if (!ok) return cudaErrorInvalidValue;
 
-  const size_t stage_bytes = (size_t)gp.kbs * ((size_t)kATileBytes + (size_t)a.n_max * 128);
-  const size_t fixed = experts_fixed_smem();
+  // ring slots: four of token rows, the rest of the shared memory for the weights (what is in
+  // flight of them sets the rate they come from HBM at; three: 2048 tokens 143 -> 156 us a
+  // layer, five or six: the same within 2 %)
+  const size_t fixed = experts_fixed_smem(), row_slot = (size_t)gp.box[0] * 128;
   const int limit = max_smem_optin();
-  int stages = (int)((limit - (int)fixed) / (int)stage_bytes);
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages < 2) return cudaErrorInvalidConfiguration;
-  gp.stages = stages;
-  gp.n_acc = 512 / a.n_max;
+  gp.b_stages = kRowStages;
+  const long left = (long)limit - (long)fixed - (long)(gp.b_stages * row_slot);
+  gp.a_stages = left < 0 ? 0 : (int)(left / kATileBytes);
+  if (gp.a_stages > kMaxStages) gp.a_stages = kMaxStages;
+  if (gp.a_stages < 2) return cudaErrorInvalidConfiguration;
+  gp.acc_cols = pow2_cols((uint32_t)a.n_max);
+  gp.n_acc = 512 / (int)gp.acc_cols;
   if (gp.n_acc > 4) gp.n_acc = 4;
-  gp.tmem_cols = pow2_cols((uint32_t)(gp.n_acc * a.n_max));
-  const size_t smem = fixed + (size_t)stages * stage_bytes;
+  gp.tmem_cols = (uint32_t)gp.n_acc * gp.acc_cols;
+  const size_t smem = fixed + (size_t)gp.a_stages * kATileBytes + gp.b_stages * row_slot;
   static int attr_dev_mask = 0;  // the dynamic smem limit is a per-device function attribute
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1200,16 +1337,13 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (dev < 31) attr_dev_mask |= 1 << dev;
   }
-  int grid = device_sm_count();
-  // block top-k with few blocks: the CTAs start while the block routing launch (one CTA
-  // per block) still runs; leave its SMs free, so that no CTA starts only when it ends
-  if (spec && a.spec_blocks <= 16 && grid > 4 * a.spec_blocks) grid -= a.spec_blocks;
+  int grid = device_sm_count() / kCluster * kCluster;
   if (grid > kMaxPersistentCtas) grid = kMaxPersistentCtas;
+  if (grid < kCluster) return cudaErrorInvalidConfiguration;
   prof_begin(DMOE_KERNEL_EXPERTS, s);
-  cudaError_t e = spec ? launch_ex(moe_experts_kernel<true>, dim3(grid), dim3(kThreads), smem, s,
-                                   !prof_serial(DMOE_KERNEL_EXPERTS), m, gp)
-                        : launch_ex(moe_experts_kernel<false>, dim3(grid), dim3(kThreads), smem,
-                                    s, !prof_serial(DMOE_KERNEL_EXPERTS), m, gp);
+  cudaError_t e = launch_cluster(spec ? moe_experts_kernel<true> : moe_experts_kernel<false>,
+                                 dim3(grid), dim3(kThreads), smem, s, kCluster,
+                                 !prof_serial(DMOE_KERNEL_EXPERTS), m, gp);
   prof_end(DMOE_KERNEL_EXPERTS, s);
   if (e != cudaSuccess) return e;
 

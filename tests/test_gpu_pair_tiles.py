@@ -1,0 +1,66 @@
+"""The general expert launch (more than 64 tokens) where its tiles can go wrong, against the CPU
+oracle: tiles of 32 to 256 token rows with remainders, blocks that fill half tiles in twos or
+fours, blocks that fill none, d and I of an odd number of 128-row tiles, more token tiles than
+one, fewer units than clusters, and gate and up weights that no single copy can bring."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from dmoe_synth import ROUTE_TOKEN, TINY
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+
+SMALL = TINY.with_(n_experts=32, top_k=4, d_ff_shared=128, bias_scale=0.5)
+CASES = {
+    # block top-k read block by block: half tiles of whole blocks (a multiple of 2 or 4 blocks)
+    "blocks_24x5": SMALL.with_(block_size=24, n_blocks=5),
+    "blocks_40x4_d384": SMALL.with_(block_size=40, n_blocks=4, d_model=384),
+    "blocks_8x33": SMALL.with_(block_size=8, n_blocks=33, n_experts=8),
+    "blocks_128x3": SMALL.with_(block_size=128, n_blocks=3),
+    "blocks_48x9_d640": SMALL.with_(block_size=48, n_blocks=9, d_model=640, n_experts=16),
+    # no half tile of whole blocks: the copied rows
+    "blocks_72x3": SMALL.with_(block_size=72, n_blocks=3),
+    "blocks_33x8_p07": SMALL.with_(block_size=33, n_blocks=8, top_p=0.7),
+    "blocks_32x10_p06_fewer": SMALL.with_(n_blocks=10, block_size=32, top_p=0.6, top_k=3,
+                                          block_top_k=4),
+    # token routing: the fewest tokens, remainders of 1 and 44 rows in a second token tile
+    "token_65_k1": SMALL.with_(block_size=13, n_blocks=5, mode=ROUTE_TOKEN, top_k=1,
+                               d_ff_shared=0),
+    "token_257_all": SMALL.with_(block_size=257, n_blocks=1, mode=ROUTE_TOKEN, n_experts=8,
+                                 top_k=8),
+    "token_300_d384_I384": SMALL.with_(block_size=60, n_blocks=5, mode=ROUTE_TOKEN, n_experts=8,
+                                       top_k=8, d_model=384, d_ff=384, d_ff_shared=256),
+}
+
+
+@pytest.mark.parametrize("name,one_tensor", [(n, False) for n in CASES] +
+                         [("blocks_24x5", True), ("token_300_d384_I384", True)])
+def test_layer_matches_oracle(name, one_tensor):
+    shape = CASES[name]
+    m = P.dm()
+    dev, host = P.make(shape, seed=7)
+    if one_tensor:   # W_up is W_gate: at distance 0 the two are not one strided tensor
+        for a, b in (("w_up", "w_gate"), ("ws_up", "ws_gate")):
+            dev[a], host[a] = dev[b], host[b]
+    from paper_2605_30876_gb300.layer import MoELayer
+    layer = MoELayer.from_shape(shape, dev)
+    y = layer.forward(dev["x"]).clone()
+    st, info = m.dmoe_get_device_error(layer.ws)
+    assert st == 0, info
+    idx = layer.topk_idx.cpu().numpy()
+    orc = P.oracle_routing(shape, host)
+    assert int(layer.n_unique.item()) == len(np.unique(idx))
+    P.check_output(y, P.oracle_output(host, idx, orc.scores), label=name)
+    assert torch.equal(y, layer.forward(dev["x"]))
+    # the same routing through the dispatch and the experts called on their own (gathered rows)
+    gate = torch.from_numpy(O.gates_for(orc.scores, idx).astype(np.float32)).cuda()
+    out, ws = P.gpu_dispatch(shape, layer.topk_idx)
+    y2 = torch.empty_like(y)
+    m.dmoe_moe_forward(layer.desc, dev["x"], dev["w_gate"], dev["w_up"], dev["w_down"],
+                       dev["ws_gate"], dev["ws_up"], dev["ws_down"], gate, out["n_unique"],
+                       out["unique_ids"], out["offsets"], out["rows"], out["pos"], y2, workspace=ws)
+    st, info = m.dmoe_get_device_error(ws)
+    assert st == 0, info
+    P.check_output(y2, P.oracle_output(host, idx, orc.scores), label=name + " experts")
