@@ -1,59 +1,56 @@
-// Dispatch of a forward in two launches over 32-token chunks (one CTA per chunk):
-//   dispatch_count_kernel  the chunk's token bitmap per expert (bits[c][e]: bit l for token
-//                          32c + l); the last CTA to finish (atomic ticket) adds the bitmaps'
-//                          counts over the chunks per expert (base[c][e] = pairs of e in
-//                          chunks before c) and scans over the experts: the offsets, the
-//                          unique list and U
-//   dispatch_place_kernel  each (token, slot) goes to row off[e] + base[c][e] + the popcount
-//                          of bits[c][e] below its token; in the fused layer call it also
-//                          copies the x rows into dispatch order (16 CTAs per chunk)
-// Every sum runs in a fixed order (no order depends on atomics), and each expert's rows are
-// ordered by token, the canonical dispatch form. An id outside [0, E) or an expert twice in
-// one token is recorded as a fault; the outputs are then unspecified (rows stay in range).
+// Dispatch of a forward over 32-token chunks:
+//   dispatch_bits_kernel   (more than 512 tokens) the chunk's token bitmap per expert
+//                          (bits[c][e]: bit l for token 32c + l), one CTA per chunk
+//   dispatch_place_kernel  every CTA finds, per expert, its pairs and those of the chunks
+//                          before its own (from the bitmaps, or from all ids itself), and by a
+//                          scan over the experts their rows' offsets; each (token, slot) of its
+//                          chunk goes to row offset[e] + pairs before the chunk + the popcount
+//                          of bits[c][e] below its token. The first CTA writes the offsets, the
+//                          unique list and U. In the fused layer call it also copies the x rows
+//                          into dispatch order (16 CTAs per chunk)
+// No launch waits for the last CTA of another (a ticket and a second phase in one CTA took 3 us):
+// the counts are cheap enough to be made in every CTA.
+// Every sum is of integers, and each expert's rows are ordered by token, the canonical
+// dispatch form. An id outside [0, E) or an expert twice in one token is recorded as a fault;
+// the outputs are then unspecified (rows stay in range).
 #include "block_reduce.cuh"
 #include "dmoe_internal.cuh"
 #include "trace_log.cuh"
-
-// Debug builds (-DDMOE_TRACE): phase times of dispatch_count_kernel (%globaltimer, ns),
-// g_dtr[cta * 16 + slot]: 0 entry, 1 ids loaded, 2 bitmap built, 3 bitmap stored, 4 ticket
-// taken; the last CTA: 5 prefix over the chunks, 6 scans, 7 outputs written.
-#ifdef DMOE_TRACE
-__device__ uint64_t g_dtr[1024 * 16];
-#define DTR_AT(slot)                                                                      \
-  do {                                                                                    \
-    if (threadIdx.x == 0) {                                                               \
-      uint64_t t_;                                                                        \
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_));                             \
-      g_dtr[(blockIdx.x % 1024) * 16 + (slot)] = t_;                                      \
-    }                                                                                     \
-  } while (0)
-#else
-#define DTR_AT(slot) ((void)0)
-#endif
 
 namespace dmoe {
 namespace {
 
 constexpr int kDispThreads = 256;
 constexpr int kDispPerThread = (32 * kMaxTopK + kDispThreads - 1) / kDispThreads;
+// Forwards of up to this many tokens take one launch: every CTA counts all T k ids itself (8 KB
+// at 256 tokens and k = 8), instead of reading bitmaps that a launch before it has written
+// (256 tokens: 9.4 us in two launches, 5.1 in one; with bitmaps, T / 32 words per expert are
+// read instead, the shorter way for large T).
+constexpr int kOneLaunchTokens = 512;
 
+// The id's bit in the chunk's bitmaps (token l of the chunk). `check`: record ids out of range
+// and experts that a token has twice.
+__device__ __forceinline__ void add_bit(uint32_t* bits, int e, int l, int E, bool check,
+                                        DevErrRecord* err, int i) {
+  if (e < 0 || e >= E) {
+    if (check) record_error(err, kErrExpertId, kAtDispatch, i);
+    return;
+  }
+  if ((atomicOr(&bits[e], 1u << l) & (1u << l)) != 0u && check)
+    record_error(err, kErrDupExpert, kAtDispatch, i);
+}
+
+// Large forwards: the chunk's token bitmap per expert.
 __global__ void __launch_bounds__(kDispThreads)
-dispatch_count_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
-                      uint32_t* __restrict__ gbits, int32_t* __restrict__ gbase,
-                      int32_t* __restrict__ goff, int32_t* __restrict__ n_unique,
-                      int32_t* __restrict__ unique_ids, int32_t* __restrict__ offsets,
-                      DevErrRecord* err, int32_t* ticket) {
+dispatch_bits_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
+                     uint32_t* __restrict__ gbits, DevErrRecord* err) {
   __shared__ uint32_t bits[kMaxExperts];
-  __shared__ int iscr[32];
-  __shared__ int s_last;
   const int c = blockIdx.x, tid = threadIdx.x;
   const int t0 = c * 32, ntok = T - t0 < 32 ? T - t0 : 32, np = ntok * k;
-  const int nchunks = gridDim.x, pairs = T * k;
   // the next launch reads the routing too: it may start once every CTA is past this wait
   pdl_wait();
   pdl_launch_dependents();
   KLOG(DMOE_KERNEL_DISPATCH, 0);
-  DTR_AT(0);
   int ids[kDispPerThread];
 #pragma unroll
   for (int j = 0; j < kDispPerThread; ++j) {
@@ -62,107 +59,114 @@ dispatch_count_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
   }
   for (int e = tid; e < E; e += kDispThreads) bits[e] = 0u;
   __syncthreads();
-  DTR_AT(1);
 #pragma unroll
   for (int j = 0; j < kDispPerThread; ++j) {
     const int p = tid + j * kDispThreads;
-    if (p >= np) continue;
-    const int i = t0 * k + p, e = ids[j];
-    if (e < 0 || e >= E) {
-      record_error(err, kErrExpertId, kAtDispatch, i);
-      continue;
-    }
-    const uint32_t bit = 1u << ((i / k) & 31);
-    if (atomicOr(&bits[e], bit) & bit) record_error(err, kErrDupExpert, kAtDispatch, i);
+    if (p < np) add_bit(bits, ids[j], p / k, E, true, err, t0 * k + p);
   }
   __syncthreads();
-  DTR_AT(2);
   for (int e = tid; e < E; e += kDispThreads) gbits[(size_t)c * E + e] = bits[e];
-  // the last CTA to get here sees every chunk's bitmap
-  __syncthreads();
-  DTR_AT(3);
-  if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(ticket, 1) == nchunks - 1 ? 1 : 0;
-  }
-  __syncthreads();
-  DTR_AT(4);
-  if (!s_last) return;
-  __threadfence();
-  int cnt = 0;
-  if (tid < E) {
-    for (int c0 = 0; c0 < nchunks; c0 += 32) {
-      uint32_t w[32];   // one round of loads per 32 chunks
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        w[j] = c0 + j < nchunks ? __ldcg(gbits + (size_t)(c0 + j) * E + tid) : 0u;
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        if (c0 + j < nchunks) {
-          gbase[(size_t)(c0 + j) * E + tid] = cnt;
-          cnt += __popc(w[j]);
-        }
-    }
-  }
-  DTR_AT(5);
-  int total_pairs = 0, n_u = 0;
-  const int off = block_exclusive_scan_i(tid < E ? cnt : 0, iscr, &total_pairs);
-  const int present = (tid < E && cnt > 0) ? 1 : 0;
-  const int upos = block_exclusive_scan_i(present, iscr, &n_u);
-  DTR_AT(6);
-  if (tid < E) {
-    goff[tid] = off;
-    if (present) {
-      unique_ids[upos] = tid;
-      offsets[upos] = off;
-    }
-  }
-  for (int u = n_u + tid; u < E; u += kDispThreads) unique_ids[u] = -1;
-  for (int u = n_u + tid; u <= E; u += kDispThreads) offsets[u] = pairs;
-  if (tid == 0) {
-    n_unique[0] = n_u;
-    if (total_pairs != pairs) record_error(err, kErrBadDispatch, kAtDispatch, total_pairs);
-    *ticket = 0;   // ready for the next call
-  }
-  DTR_AT(7);
   KLOG(DMOE_KERNEL_DISPATCH, 1);
 }
 
 // Placement of chunk blockIdx.x; with xperm, blockIdx.y takes its share of the chunk's
 // (token, slot) pairs and also copies their x rows into dispatch order (kGatherRows rows
-// in flight per thread).
+// in flight per thread). Every CTA finds the experts' row offsets and the rows of the chunks
+// before its own: from the chunks' bitmaps, or (kOneLaunch) from all ids.
 constexpr int kPlaceSplit = 16;    // CTAs per chunk when the rows are copied too
 constexpr int kGatherRows = 8;
+template <bool kOneLaunch>
 __global__ void __launch_bounds__(kDispThreads)
 dispatch_place_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
-                      const uint32_t* __restrict__ gbits, const int32_t* __restrict__ gbase,
-                      const int32_t* __restrict__ goff, int32_t* __restrict__ rows,
-                      int32_t* __restrict__ pos, const __nv_bfloat16* __restrict__ x,
-                      __nv_bfloat16* __restrict__ xperm, int d, int32_t* zero, int n_zero) {
+                      const uint32_t* __restrict__ gbits, int32_t* __restrict__ n_unique,
+                      int32_t* __restrict__ unique_ids, int32_t* __restrict__ offsets,
+                      int32_t* __restrict__ rows, int32_t* __restrict__ pos,
+                      const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ xperm,
+                      int d, int32_t* zero, int n_zero, DevErrRecord* err) {
   __shared__ uint32_t bits[kMaxExperts];
   __shared__ int base[kMaxExperts];
+  __shared__ int iscr[32];
   __shared__ int s_r[32 * kMaxTopK], s_t[32 * kMaxTopK];
-  const int c = blockIdx.x, tid = threadIdx.x;
+  const int c = blockIdx.x, tid = threadIdx.x, nchunks = gridDim.x;
   const int t0 = c * 32, ntok = T - t0 < 32 ? T - t0 : 32, np = ntok * k;
   const int pairs = T * k;
+  const bool first = c == 0 && blockIdx.y == 0;
   // this CTA's pairs of the chunk
   const int per = (np + gridDim.y - 1) / gridDim.y;
   const int p0 = blockIdx.y * per, p1 = p0 + per < np ? p0 + per : np;
-  // the routing was complete before the counting launch let this one start
+  pdl_wait();
+  // The next launch may start; the first CTA lets it only once the unique list is written (the
+  // expert launch reads it before its own dependency wait).
+  if (!first) pdl_launch_dependents();
+  KLOG(7, 0);
   int ids[kDispPerThread];
 #pragma unroll
   for (int j = 0; j < kDispPerThread; ++j) {
     const int p = p0 + tid + j * kDispThreads;
     ids[j] = p < p1 ? __ldcg(topk_idx + t0 * k + p) : 0;
   }
-  pdl_wait();
-  pdl_launch_dependents();   // after the wait: a waiting dependent would share the SMs
-  KLOG(7, 0);
-  if (zero != nullptr && blockIdx.x == 0 && blockIdx.y == 0)
-    for (int i = tid; i < n_zero; i += kDispThreads) zero[i] = 0;
-  for (int e = tid; e < E; e += kDispThreads) {
-    bits[e] = gbits[(size_t)c * E + e];
-    base[e] = gbase[(size_t)c * E + e] + goff[e];
+  // pairs per expert, and those in the chunks before this one
+  int cnt = 0, before = 0;
+  if (kOneLaunch) {
+    base[tid] = 0;
+    bits[tid] = 0u;
+    __syncthreads();
+    const bool check = blockIdx.y == 0;
+    for (int i0 = 0; i0 < pairs; i0 += 8 * kDispThreads) {
+      int e[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = i0 + tid + j * kDispThreads;
+        e[j] = i < pairs ? __ldcg(topk_idx + i) : -1;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int i = i0 + tid + j * kDispThreads, p = i - t0 * k;
+        if (p >= 0 && p < np) add_bit(bits, e[j], p / k, E, check, err, i);
+        // (at most 512 * 16 pairs: both counts fit one word)
+        if (e[j] >= 0 && e[j] < E) atomicAdd(&base[e[j]], p < 0 ? 0x10001 : 1);
+      }
+    }
+    __syncthreads();
+    cnt = base[tid] & 0xffff;
+    before = base[tid] >> 16;
+  } else if (tid < E) {
+    bits[tid] = __ldcg(gbits + (size_t)c * E + tid);
+    for (int c0 = 0; c0 < nchunks; c0 += 32) {
+      uint32_t w[32];   // one round of loads per 32 chunks
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        w[j] = c0 + j < nchunks ? __ldcg(gbits + (size_t)(c0 + j) * E + tid) : 0u;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int n = __popc(w[j]);
+        cnt += n;
+        before += c0 + j < c ? n : 0;
+      }
+    }
+  }
+  int total_pairs = 0;
+  const int off = block_exclusive_scan_i(cnt, iscr, &total_pairs);
+  base[tid] = off + before;
+  if (first) {
+    int n_u = 0;
+    const int present = cnt > 0 ? 1 : 0;
+    const int upos = block_exclusive_scan_i(present, iscr, &n_u);
+    if (present) {
+      unique_ids[upos] = tid;
+      offsets[upos] = off;
+    }
+    for (int u = n_u + tid; u < E; u += kDispThreads) unique_ids[u] = -1;
+    for (int u = n_u + tid; u <= E; u += kDispThreads) offsets[u] = pairs;
+    if (tid == 0) {
+      n_unique[0] = n_u;
+      if (total_pairs != pairs) record_error(err, kErrBadDispatch, kAtDispatch, total_pairs);
+    }
+    __threadfence();
+    __syncthreads();
+    pdl_launch_dependents();
+    if (zero != nullptr)
+      for (int i = tid; i < n_zero; i += kDispThreads) zero[i] = 0;
   }
   __syncthreads();
 #pragma unroll
@@ -206,21 +210,25 @@ dispatch_place_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
 
 }  // namespace
 
+int dispatch_launches(int T) { return T <= kOneLaunchTokens ? 1 : 2; }
+
 cudaError_t launch_dispatch(const DispatchArgs& a, cudaStream_t s) {
-  if (a.bits == nullptr || a.base == nullptr || a.off == nullptr || a.ticket == nullptr ||
-      a.k > kMaxTopK || a.E > kMaxExperts || (a.xperm != nullptr && (a.x == nullptr || a.d % 8)))
+  if (a.bits == nullptr || a.k > kMaxTopK || a.E > kMaxExperts ||
+      (a.xperm != nullptr && (a.x == nullptr || a.d % 8)))
     return cudaErrorInvalidValue;
   const int nchunks = (a.T + 31) / 32;
+  const bool one = dispatch_launches(a.T) == 1;
   prof_begin(DMOE_KERNEL_DISPATCH, s);
-  cudaError_t e = launch_ex(dispatch_count_kernel, dim3(nchunks), dim3(kDispThreads), 0, s, true,
-                            a.topk_idx, a.T, a.E, a.k, a.bits, a.base, a.off, a.n_unique,
-                            a.unique_ids, a.offsets, a.err, a.ticket);
+  cudaError_t e = cudaSuccess;
+  if (!one)
+    e = launch_ex(dispatch_bits_kernel, dim3(nchunks), dim3(kDispThreads), 0, s, true, a.topk_idx,
+                  a.T, a.E, a.k, a.bits, a.err);
   if (e == cudaSuccess)
-    e = launch_ex(dispatch_place_kernel, dim3(nchunks, a.xperm != nullptr ? kPlaceSplit : 1),
-                  dim3(kDispThreads), 0, s, true, a.topk_idx, a.T, a.E, a.k,
-                  static_cast<const uint32_t*>(a.bits), static_cast<const int32_t*>(a.base),
-                  static_cast<const int32_t*>(a.off), a.rows, a.pos, a.x, a.xperm, a.d, a.zero,
-                  a.n_zero);
+    e = launch_ex(one ? dispatch_place_kernel<true> : dispatch_place_kernel<false>,
+                  dim3(nchunks, a.xperm != nullptr ? kPlaceSplit : 1), dim3(kDispThreads), 0, s,
+                  true, a.topk_idx, a.T, a.E, a.k, static_cast<const uint32_t*>(a.bits),
+                  a.n_unique, a.unique_ids, a.offsets, a.rows, a.pos, a.x, a.xperm, a.d, a.zero,
+                  a.n_zero, a.err);
   prof_end(DMOE_KERNEL_DISPATCH, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -230,7 +238,4 @@ cudaError_t launch_dispatch(const DispatchArgs& a, cudaStream_t s) {
 
 #ifdef DMOE_TRACE
 DMOE_KLOG_EXPORT(dmoe_debug_klog_dispatch)
-extern "C" int dmoe_debug_dtr(void* host) {
-  return (int)cudaMemcpyFromSymbol(host, g_dtr, sizeof(g_dtr));
-}
 #endif

@@ -138,8 +138,6 @@ Workspace plan_workspace(const dmoe_layer_desc& d) {
                     : 0);
   const size_t nchunks = (T + 31) / 32;
   w.disp_bits = take(sizeof(uint32_t) * nchunks * E);
-  w.disp_base = take(sizeof(int32_t) * nchunks * E);
-  w.disp_off = take(sizeof(int32_t) * E);
   w.w_parts_bytes = tc ? router_tc_parts_bytes((int)dm, (int)E) : 0;
   w.w_parts = take(w.w_parts_bytes);
   w.tc_part = take(sizeof(float) * (size_t)w.tc_splits * T * E);
@@ -189,9 +187,6 @@ T* at(void* ws, size_t off) {
 
 void set_dispatch_scratch(DispatchArgs* a, void* ws, const Workspace& plan) {
   a->bits = at<uint32_t>(ws, plan.disp_bits);
-  a->base = at<int32_t>(ws, plan.disp_base);
-  a->off = at<int32_t>(ws, plan.disp_off);
-  a->ticket = at<int32_t>(ws, plan.tickets) + kDispatchTicket;
 }
 
 dmoe_status cuda_status(cudaError_t e) {
@@ -574,14 +569,15 @@ int32_t dmoe_layer_forward_launches(const dmoe_layer_desc* desc) {
     n += 2;                                                   // logits, softmax / top-k
     n += router_tc_ok(T, desc->d_model, desc->n_experts) ? 1 : 0;   // the split of W_r
     n += desc->mode == DMOE_ROUTE_BLOCK ? 1 : 0;              // Algorithm 1
-    n += 2;                                                   // dispatch: count, place
+    n += dispatch_launches(T);                                // dispatch: (bitmaps,) place
   }
   // experts and combine; the general experts' gather is a launch of its own only after the
   // fused routing launch (otherwise the dispatch placement does it); with block top-k on the
   // general path the expert launch does the dispatch (no dispatch launches)
   const bool dec = experts_decode_ok(T, desc->d_model, desc->d_ff, desc->d_ff_shared);
   const bool cluster = route_cluster_ok(T, desc->d_model, desc->n_experts);
-  if (!cluster && !dec && experts_spec_ok(*desc, expert_n_max(*desc))) n -= 2;
+  if (!cluster && !dec && experts_spec_ok(*desc, expert_n_max(*desc)))
+    n -= dispatch_launches(T);
   n += (!dec && cluster) ? 3 : 2;
   return n;
 }

@@ -81,8 +81,6 @@ struct Workspace {
   size_t spec;         // int32 [n_blocks, k]: the coreset of every block (block top-k call)
                        // (decode-size forwards only)
   size_t disp_bits;    // u32 [ceil(T/32), E]: dispatch, token bitmap per (32-token chunk, expert)
-  size_t disp_base;    // int32 [ceil(T/32), E]: dispatch, pairs of the expert in earlier chunks
-  size_t disp_off;     // int32 [E]: dispatch, first row of every expert (all experts)
   size_t w_parts;      // bf16 [3E, d]: split of W_r for the tcgen05 router (large forwards)
   size_t w_parts_bytes;
   size_t tc_part;      // fp32 [tc_splits, T, E]: the tcgen05 router's partial logits
@@ -209,11 +207,7 @@ struct DispatchArgs {
   int32_t* pos;
   int T, E, k;
   DevErrRecord* err;
-  // scratch of the multi-CTA dispatch (Workspace::disp_*) and its ticket (zero between calls)
-  uint32_t* bits;
-  int32_t* base;
-  int32_t* off;
-  int32_t* ticket;
+  uint32_t* bits;   // scratch (Workspace::disp_bits)
   // optional (the fused layer call of the general path): the placement also copies x's
   // rows into dispatch order (xperm [T*k, d]) and clears zero[0 .. n_zero) (the expert
   // launch's tile counters), so that the expert launch needs no gather launch
@@ -223,8 +217,8 @@ struct DispatchArgs {
   int32_t* zero;
   int n_zero;
 };
-// ticket index (in Workspace::tickets) of the dispatch launch
-constexpr int kDispatchTicket = 1;
+// launches of a dispatch of T tokens
+int dispatch_launches(int T);
 cudaError_t launch_dispatch(const DispatchArgs& a, cudaStream_t s);
 
 // Routing of one forward. With `dsp` set, the dispatch is computed too (inside the fused

@@ -191,13 +191,12 @@ __device__ uint64_t g_trace[kMaxPersistentCtas * 64];
 // tile); the shared expert's group comes first in both lists. A cluster's first unit is its
 // number; it takes every further one from a global counter when it begins to load the one
 // before (units differ in cost, and a fixed share left the last cluster 12-20 us behind the
-// first at 256 to 2048 tokens). A
-// cluster's unit numbers ascend, so its gate/up units precede its down units and a gate/up
-// unit never waits on another unit. The weights of a down unit are loaded as ring slots free;
-// only its token rows wait (bounded) for the gate/up tiles of those rows to be published
-// (h_ready), so weight streaming of both phases overlaps. kSpec: the block
-// top-k form (GemmParams::spec_words), compiled separately so that the other form carries
-// none of its code.
+// first at 256 to 2048 tokens). A cluster's unit numbers ascend, so its gate/up units precede
+// its down units and a gate/up unit never waits on another unit. The weights of a down unit are
+// loaded as ring slots free; only its token rows wait (bounded) for the gate/up tiles of those
+// rows to be published (h_ready), so weight streaming of both phases overlaps. kSpec: the block
+// top-k form (GemmParams::spec_words), compiled separately so that the other form carries none
+// of its code.
 template <bool kSpec>
 __global__ void __launch_bounds__(kThreads, 1)
 moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
@@ -278,11 +277,11 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   }
   ptx::cluster_arrive();   // the barriers of both CTAs are set up
   ptx::cluster_wait();
-  // No dependency wait here. The launch before this one (the dispatch placement or the gather)
-  // released it after its own wait, so the unique list and the offsets are complete; what that
-  // launch itself writes (the rows in dispatch order, the zeroed counters) is used by the row
-  // producer, the plan warp's polls and the unit counter, which wait first. The weights of the
-  // first unit are on their way by then.
+  // No dependency wait here. The launch before this one released it once the unique list and
+  // the offsets were written and visible (the dispatch placement), or after its own wait for the
+  // launch that wrote them (the gather); what it writes besides (the rows in dispatch order, the
+  // zeroed counters) is used by the row producer, the plan warp's polls and the unit counter,
+  // which wait first. The weights of the first unit are on their way by then.
 
   // Enters the cluster's unit i >= 1 into the queue of both CTAs (one thread of the first CTA;
   // the entry's last unit must have been read by both).
@@ -375,7 +374,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       }
       __syncwarp();
     } else {
-      U = *p.n_unique;
+      U = __ldcg(p.n_unique);
       if (U < 0 || U > p.E) {
         if (lane == 0) record_error(p.err, kErrBadDispatch, kAtGateUp, U);
         U = 0;
@@ -395,9 +394,9 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
           e = g_e[g];
           Ig = g < U ? p.I : p.Is;
         } else if (g < U) {
-          row0 = p.offsets[g];
-          cnt = p.offsets[g + 1] - row0;
-          e = p.unique_ids[g];
+          row0 = __ldcg(p.offsets + g);
+          cnt = __ldcg(p.offsets + g + 1) - row0;
+          e = __ldcg(p.unique_ids + g);
           Ig = p.I;
           if (e < 0 || e >= p.E || cnt < 0 || cnt > p.T || row0 < 0 ||
               row0 + cnt > p.T * p.k) {
@@ -462,7 +461,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     const int total = (int)(3 * per * U);
     if (pf.bytes * U <= kDownPrefetchMax)
       for (int c = (int)(2 * per * U) + blockIdx.x; c < total; c += gridDim.x)
-        l2_prefetch_chunk(pf, spec ? g_e : p.unique_ids, U, c);
+        l2_prefetch_chunk(pf, g_e, U, c);
     if (p.ws_gate != nullptr) {
       L2Prefetch sp;
       sp.ptr[0] = p.ws_gate;
