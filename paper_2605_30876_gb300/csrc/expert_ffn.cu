@@ -58,7 +58,6 @@ constexpr uint64_t kWaitTimeoutNs = 1000000000ull;  // 1 s
 constexpr int kMaxStages = 12;                     // ring slots of the weights, at most
 constexpr int kRowStages = 4;                      // ring slots of the token rows
 constexpr int kProgress = 64;                      // steps (K = 128) whose completion is remembered
-constexpr int64_t kDownPrefetchMax = (int64_t)64 << 20;   // half of the 129 MB L2
 constexpr int kQueue = 4;                          // units handed out and not yet taken up by every role
 constexpr int kSpecBlocks = 64;                    // blocks of a block top-k forward, at most
 constexpr int kSpecPairs = kSpecBlocks * kMaxTopK;   // (block, coreset member) pairs, at most
@@ -75,7 +74,6 @@ struct GemmParams {
   int32_t* h_ready;       // [(E+1) * ntiles]: gate/up tiles done per (group, token tile)
   int32_t* next_unit;     // units handed out beyond every cluster's first
   DevErrRecord* err;
-  const void* w_down;     // routed W_down, prefetched into L2 for the unique experts
   const void* ws_gate; const void* ws_up; const void* ws_down;  // shared, prefetched if set
   int T, d, E, k, I, Is;
   int n_max;              // token tile, at most; a multiple of
@@ -448,29 +446,17 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   const int G = s_sched[0], U = s_sched[1], n_gu = s_sched[2], n_dn = s_sched[3];
   const int units = n_gu + n_dn;
   if (tid == 0) DMOE_TRACE_AT(1);
-  if (tid == 64) {
-    // Pull the down-projection weights of every unique expert into L2 now, spread over all
-    // CTAs: the down units of the second wave then read them from L2, and HBM keeps
-    // streaming while the gate/up results are produced and published. Only while they
-    // fit in half of L2: beyond that the prefetched lines are evicted before their use
-    // and only add HBM traffic (token routing at 2048 tokens: 256 experts, 537 MB).
-    L2Prefetch pf;
-    pf.ptr[2] = p.w_down;
-    pf.bytes = (int64_t)p.d * p.I * 2;
-    const int64_t per = (pf.bytes + kPrefetchChunk - 1) / kPrefetchChunk;
-    const int total = (int)(3 * per * U);
-    if (pf.bytes * U <= kDownPrefetchMax)
-      for (int c = (int)(2 * per * U) + blockIdx.x; c < total; c += gridDim.x)
-        l2_prefetch_chunk(pf, g_e, U, c);
-    if (p.ws_gate != nullptr) {
-      L2Prefetch sp;
-      sp.ptr[0] = p.ws_gate;
-      sp.ptr[1] = p.ws_up;
-      sp.ptr[2] = p.ws_down;
-      sp.bytes = (int64_t)p.d * p.Is * 2;
-      const int sper = (int)((sp.bytes + kPrefetchChunk - 1) / kPrefetchChunk);
-      for (int c = blockIdx.x; c < 3 * sper; c += gridDim.x) l2_prefetch_chunk(sp, nullptr, 1, c);
-    }
+  // (No L2 prefetch of the routed weights: the units' own loads keep HBM busy, and W_down pulled
+  // into L2 at this point competed with the gate/up stream that the down units wait for
+  // anyway: 256 tokens 51.1 us a layer without it, 55.4 with it; 5 x 60 tokens 65.4 and 70.7.)
+  if (tid == 64 && p.ws_gate != nullptr) {
+    L2Prefetch sp;
+    sp.ptr[0] = p.ws_gate;
+    sp.ptr[1] = p.ws_up;
+    sp.ptr[2] = p.ws_down;
+    sp.bytes = (int64_t)p.d * p.Is * 2;
+    const int sper = (int)((sp.bytes + kPrefetchChunk - 1) / kPrefetchChunk);
+    for (int c = blockIdx.x; c < 3 * sper; c += gridDim.x) l2_prefetch_chunk(sp, nullptr, 1, c);
   }
 
   // A unit: phase, group, m tile, n tile, rows of the token tile. The plan warp finds it from
@@ -1259,7 +1245,6 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   gp.h_ready = a.h_ready;
   gp.next_unit = a.h_ready + n_ready - 1;
   gp.err = a.err;
-  gp.w_down = a.w_down;
   if (has_shared && a.prefetch_shared) {
     gp.ws_gate = a.ws_gate;
     gp.ws_up = a.ws_up;
