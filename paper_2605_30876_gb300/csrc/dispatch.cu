@@ -218,8 +218,11 @@ cudaError_t launch_dispatch(const DispatchArgs& a, cudaStream_t s) {
     return cudaErrorInvalidValue;
   const int nchunks = (a.T + 31) / 32;
   const bool one = dispatch_launches(a.T) == 1;
+  static std::atomic<uint32_t> carveout[2];
+  cudaError_t e = one ? max_shared_carveout(dispatch_place_kernel<true>, carveout[1])
+                      : max_shared_carveout(dispatch_place_kernel<false>, carveout[0]);
+  if (e != cudaSuccess) return e;
   prof_begin(DMOE_KERNEL_DISPATCH, s);
-  cudaError_t e = cudaSuccess;
   if (!one)
     e = launch_ex(dispatch_bits_kernel, dim3(nchunks), dim3(kDispThreads), 0, s, true, a.topk_idx,
                   a.T, a.E, a.k, a.bits, a.err);

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/dmoe.h"
 
 namespace dmoe {
@@ -353,6 +355,22 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Lets a CTA of the expert launch (which takes nearly all shared memory of an SM) start on an SM
+// where a CTA of `kernel` still runs: an SM's split between L1 and shared memory changes only
+// while it is empty, so the small kernels before the expert launch ask for the largest shared
+// part too. Once per device and kernel (`done`: a bit per device).
+template <typename F>
+inline cudaError_t max_shared_carveout(F* kernel, std::atomic<uint32_t>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  const uint32_t bit = dev < 32 ? 1u << dev : 0u;
+  if (e != cudaSuccess || (done.load(std::memory_order_relaxed) & bit) != 0u) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
 }
 
 // host helpers

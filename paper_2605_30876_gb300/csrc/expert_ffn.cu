@@ -56,7 +56,7 @@ constexpr int kLevels = 3;                         // heights of the token row b
 constexpr int kMaxGroups = kMaxExperts + 1;
 constexpr uint64_t kWaitTimeoutNs = 1000000000ull;  // 1 s
 constexpr int kMaxStages = 12;                     // ring slots of the weights, at most
-constexpr int kRowStages = 4;                      // ring slots of the token rows
+constexpr int kRowStages = 5;                      // ring slots of the token rows
 constexpr int kProgress = 64;                      // steps (K = 128) whose completion is remembered
 constexpr int kQueue = 4;                          // units handed out and not yet taken up by every role
 constexpr int kSpecBlocks = 64;                    // blocks of a block top-k forward, at most
@@ -1228,8 +1228,11 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   //    routing launch has cleared them and the token rows are read from x by block)
   if (!a.gathered && !spec) {
     const int grid = pairs < 1024 ? pairs : 1024;
+    static std::atomic<uint32_t> carveout;
+    cudaError_t e = max_shared_carveout(gather_kernel, carveout);
+    if (e != cudaSuccess) return e;
     prof_begin(DMOE_KERNEL_GATHER, s);
-    cudaError_t e = launch_ex(gather_kernel, dim3(grid), dim3(256), 0, s, true, a.x, a.rows,
+    e = launch_ex(gather_kernel, dim3(grid), dim3(256), 0, s, true, a.x, a.rows,
                               a.xperm, a.h_ready, n_ready, pairs, a.k, a.d);
     prof_end(DMOE_KERNEL_GATHER, s);
     if (e != cudaSuccess) return e;
@@ -1294,15 +1297,19 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   }
   if (!ok) return cudaErrorInvalidValue;
 
-  // ring slots: four of token rows, the rest of the shared memory for the weights (what is in
-  // flight of them sets the rate they come from HBM at; three: 2048 tokens 143 -> 156 us a
-  // layer, five or six: the same within 2 %)
+  // ring slots: five of token rows, the rest of the shared memory for the weights (what is in
+  // flight of them sets the rate they come from HBM at). Four / five / six, us per layer: 256
+  // tokens 51.8 / 50.6 / 50.1 (block top-k) and 79.9 / 79.0 / 79.8 (p = 0.6), 1024 tokens with
+  // p = 0.6 136 / 134 / 136, 2048 tokens with token routing 320 / 315 / 324
   const size_t fixed = experts_fixed_smem(), row_slot = (size_t)gp.box[0] * 128;
   const int limit = max_smem_optin();
   gp.b_stages = kRowStages;
   const long left = (long)limit - (long)fixed - (long)(gp.b_stages * row_slot);
   gp.a_stages = left < 0 ? 0 : (int)(left / kATileBytes);
-  if (gp.a_stages > kMaxStages) gp.a_stages = kMaxStages;
+  // (block top-k: room for a CTA of the block routing launch beside this launch's, which
+  // start while it runs)
+  const int most = spec ? kMaxStages - 4 : kMaxStages;
+  if (gp.a_stages > most) gp.a_stages = most;
   if (gp.a_stages < 2) return cudaErrorInvalidConfiguration;
   gp.acc_cols = pow2_cols((uint32_t)a.n_max);
   gp.n_acc = 512 / (int)gp.acc_cols;

@@ -179,6 +179,9 @@ cudaError_t launch_router(const RouterArgs& a, const DispatchArgs* dsp, int32_t*
                   a.probs, a.probs_hat, a.topk_idx, a.topk_gate, a.T, a.E, a.kb, a.mode);
     if (e != cudaSuccess) return e;
     if (a.mode == DMOE_ROUTE_BLOCK) {
+      static std::atomic<uint32_t> carveout;
+      e = max_shared_carveout(block_route_kernel, carveout);
+      if (e != cudaSuccess) return e;
       e = launch_ex(block_route_kernel, dim3(a.n_blocks), dim3(256), 0, s, true, a.probs,
                     a.probs_hat, a.E, a.kb, a.k, a.B, a.top_p, a.topk_idx, a.topk_gate, a.coreset,
                     a.coreset_size, a.spec_words, a.ready_clear, a.n_ready_clear);
