@@ -86,8 +86,16 @@ typedef struct {
 
 /* Bytes of device workspace needed by every call below for this shape (host only; no
  * CUDA call). One workspace sized for the desc serves all calls on that desc. A workspace
- * must be zero-filled once before its first use; every call leaves it reusable. */
+ * must be zero-filled once before its first use (dmoe_workspace_init); every call leaves it
+ * reusable. */
 dmoe_status dmoe_workspace_size(const dmoe_layer_desc* desc, size_t* bytes /* host */);
+
+/* Zero-fills a workspace (asynchronously, on `stream`) and forgets on the host that a workspace
+ * at this address was prepared (dmoe_router_prepare). New memory at an address that a prepared
+ * workspace had before has to come through this call, or be prepared again, before its first
+ * use: zero-filled in another way it would be taken for the prepared one.
+ *   workspace                256-byte aligned device memory; bytes: its size */
+dmoe_status dmoe_workspace_init(void* workspace, size_t bytes, void* stream);
 
 /* Router and routing — §4.2 (s_i = Router(t_i); S_block = aggregation of the s_i;
  * C = Top-P(S~_block, p)) and Algorithm 1 (TopKMask, sum, Normalize, TopP,

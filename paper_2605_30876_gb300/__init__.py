@@ -16,7 +16,7 @@ import torch
 
 __all__ = [
     "DMOE_ROUTE_TOKEN", "DMOE_ROUTE_BLOCK", "DmoeError", "LayerDesc", "make_desc",
-    "dmoe_workspace_size", "dmoe_router", "dmoe_dispatch", "dmoe_moe_forward",
+    "dmoe_workspace_size", "dmoe_workspace_init", "dmoe_router", "dmoe_dispatch", "dmoe_moe_forward",
     "dmoe_layer_forward", "dmoe_get_device_error", "dmoe_status_string", "dmoe_abi_version",
     "dmoe_layer_forward_launches",
     "alloc_workspace", "LIB_PATH", "dmoe_set_profile_events", "KERNELS",
@@ -74,6 +74,8 @@ def _load() -> ctypes.CDLL:
     st = ctypes.c_int
     lib.dmoe_workspace_size.argtypes = [D, ctypes.POINTER(ctypes.c_size_t)]
     lib.dmoe_workspace_size.restype = st
+    lib.dmoe_workspace_init.argtypes = [P, ctypes.c_size_t, P]
+    lib.dmoe_workspace_init.restype = st
     lib.dmoe_router.argtypes = [D, P, P, P, P, P, P, P, P, P, ctypes.c_size_t, P]
     lib.dmoe_router.restype = st
     lib.dmoe_router_prepare.argtypes = [D, P, P, ctypes.c_size_t, P]
@@ -155,7 +157,16 @@ def dmoe_workspace_size(desc: LayerDesc) -> int:
 
 def alloc_workspace(desc: LayerDesc, device="cuda") -> torch.Tensor:
     """A zeroed uint8 device buffer of dmoe_workspace_size(desc) bytes (torch allocates)."""
-    return torch.zeros(dmoe_workspace_size(desc), dtype=torch.uint8, device=device)
+    ws = torch.empty(dmoe_workspace_size(desc), dtype=torch.uint8, device=device)
+    dmoe_workspace_init(ws)
+    return ws
+
+
+def dmoe_workspace_init(workspace, stream=None) -> None:
+    """Zero-fills a workspace and forgets any preparation of an earlier one at its address."""
+    ws, nb = _ws(workspace)
+    with torch.cuda.device(workspace.device):
+        _check(_lib.dmoe_workspace_init(ws, nb, _stream(stream)), "dmoe_workspace_init")
 
 
 def dmoe_router(desc, x, w_r, bias, topk_idx, topk_gate, coreset=None, coreset_size=None,

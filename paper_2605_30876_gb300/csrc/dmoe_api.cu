@@ -328,6 +328,16 @@ dmoe_status dmoe_workspace_size(const dmoe_layer_desc* desc, size_t* bytes) {
   return DMOE_OK;
 }
 
+dmoe_status dmoe_workspace_init(void* workspace, size_t bytes, void* stream) {
+  if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0)
+    return DMOE_ERR_INVALID_ARG;
+  {
+    std::lock_guard<std::mutex> lock(g_prep_mu);
+    g_prep.erase(workspace);
+  }
+  return cuda_status(cudaMemsetAsync(workspace, 0, bytes, static_cast<cudaStream_t>(stream)));
+}
+
 dmoe_status dmoe_router(const dmoe_layer_desc* desc, const void* x, const float* w_r,
                         const float* bias, int32_t* topk_idx, float* topk_gate,
                         int32_t* coreset, int32_t* coreset_size, float* probs,
