@@ -47,8 +47,7 @@ constexpr int kABox = kTileM * 128;             // 128 rows x 128 B (W_down)
 constexpr int kAStage = kKB * kABox;            // 32 KB of weights in every stage
 constexpr int kMaxKBG = 4;                      // K boxes per gate/up stage (hg = 32)
 constexpr int kMaxStagesD = 6;
-constexpr int kXStride = 17;                    // floats per row of the SwiGLU exchange
-constexpr int kXchgBytes = 2 * 64 * kXStride * 4;
+constexpr int kGateRows = 8;                    // rows of W_gate, then of W_up, in an A tile
 constexpr uint64_t kTimeoutNs = 1000000000ull;  // 1 s
 constexpr int kMaxTok = 64;                     // tokens of a decode-sized forward
 
@@ -92,19 +91,22 @@ struct DParams {
   int ring_bytes;            // pipeline ring (multiple of 1 KB)
   int h32_ok;                // 32-row gate/up units allowed (d % 256 == 0, >= 3 slots fit)
   int has_shared;
+  int gu_box, sgu_box;       // gate and up rows come in one box (DMaps::gu ..): 1: gate first, 2:
+                             // up first; 0: a box per 8 rows (routed experts, shared expert)
   int n_acc;                 // TMEM accumulators of n_pad columns
   uint32_t tmem_cols;
 };
 
+// Every map sees its matrix as [K / 64][rows][64], so that one copy brings a whole stage (several
+// 64-column K boxes): the producer issues two copies per stage, weights and token rows.
 struct DMaps {
-  CUtensorMap wg, wu, wd;    // routed: [E*I, d] (64-row boxes) x2, [E*d, I] (128-row boxes)
-  CUtensorMap sg, su, sd;    // shared: [Is, d] x2, [d, Is]
-  CUtensorMap wg32, wu32;    // routed gate/up, 32-row boxes
-  CUtensorMap sg32, su32;    // shared gate/up, 32-row boxes
-  CUtensorMap x;             // x [T, d], n_pad-row boxes (rows >= T read as zeros)
-  CUtensorMap h;             // hdense, n_pad-row boxes, 128-B swizzle (down B operand)
+  CUtensorMap gu, sgu;       // gate/up, [K / 64][rows / 8][2][8][64]: 64 rows of each (K = 128)
+  CUtensorMap gu32, sgu32;   // ... 32 rows of each (K = 256)
+  CUtensorMap wg, wu, sg, su;   // ... 8 rows of one (K = 64)
+  CUtensorMap wd, sd;        // down: 128 rows, K = 128
+  CUtensorMap x, x32;        // x [T, d]: n_pad rows (rows >= T read as zeros), K = 128 / 256
+  CUtensorMap h;             // hdense: n_pad rows, K = 128 (down B operand)
   CUtensorMap hst;           // hdense, 32 columns x n_pad rows, no swizzle (tile stores)
-  CUtensorMap ys, ysh;       // yslot [T*k, d], yshared [T, d] fp32: 128 columns x 8 rows
 };
 
 // One group of the forward.
@@ -117,8 +119,6 @@ struct Grp {
 };
 
 using ptx::bulk_commit_wait_all;
-using ptx::bulk_commit_wait_read;
-using ptx::bulk_store;
 using ptx::epi_all;
 using ptx::fence_proxy_async_global;
 using ptx::ld_acquire;
@@ -129,6 +129,25 @@ using ptx::tma_store_2d;
 // silu with the fast divide: H is rounded to bf16 right after
 __device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __expf(-z)); }
 
+// One gate/up stage's weights: hg (32 or 64) rows of W_gate and the same rows of W_up from row
+// arow, 8 of each in turn, over the 64-column K boxes from kb on (32 KB).
+__device__ __forceinline__ void load_gate_up(const DMaps& tm, const DParams& p, uint8_t* dst,
+                                             uint64_t* bar, bool shared, bool h32, int arow, int kb,
+                                             uint64_t pol) {
+  if ((shared ? p.sgu_box : p.gu_box) != 0) {
+    const CUtensorMap* m = shared ? (h32 ? &tm.sgu32 : &tm.sgu) : (h32 ? &tm.gu32 : &tm.gu);
+    ptx::tma_load_5d(dst, m, bar, 0, 0, 0, arow / kGateRows, kb, pol);
+    return;
+  }
+  const int hg = h32 ? 32 : 64;
+  for (int b = 0; b < kTileM / hg; ++b)
+    for (int r = 0; r < hg; r += kGateRows, dst += 2 * kGateRows * 128) {
+      ptx::tma_load_3d(dst, shared ? &tm.sg : &tm.wg, bar, 0, arow + r, kb + b, pol);
+      ptx::tma_load_3d(dst + kGateRows * 128, shared ? &tm.su : &tm.wu, bar, 0, arow + r, kb + b,
+                       pol);
+    }
+}
+
 // kMask: the coresets are published as masks (DParams::spec_mask), compiled separately so
 // that the launch on ids carries none of that code
 template <bool kMask>
@@ -138,14 +157,12 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
   uint8_t* smem = smem_raw + ((1024u - (ptx::smem_addr(smem_raw) & 1023u)) & 1023u);
   const int bbox = p.n_pad * 128;                 // one K box of token rows
   const int bstage = kKB * bbox;                  // B bytes of a down stage
-  const int SP = p.n_pad + 1;                     // floats per row of the down staging tile
   // ring of S slots [32 KB of weights | token boxes]; S and the slot size follow hg below
   uint8_t* ring = smem;
-  // staging: a gate/up tile's H box, or a down tile as [token][128 rows] fp32 (128 x SP floats)
-  float* stage_t = reinterpret_cast<float*>(ring + p.ring_bytes);
-  float* xchg = stage_t + kTileM * SP;
-  int* tok = reinterpret_cast<int*>(xchg + 2 * 64 * kXStride);      // [kMaxTok]
-  uint64_t* full = reinterpret_cast<uint64_t*>(tok + kMaxTok);
+  uint8_t* hbox = ring + p.ring_bytes;            // staging: a gate/up tile's H box
+  int* s_row = reinterpret_cast<int*>(hbox + 2 * 64 * p.n_pad);   // [kMaxTok]: the output row of
+                                                  // a token's column in a down tile, -1: none
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_row + kMaxTok);
   uint64_t* empty = full + kMaxStagesD;
   uint64_t* acc_full = empty + kMaxStagesD;
   uint64_t* acc_empty = acc_full + 4;
@@ -175,9 +192,9 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     *s_abort = 0;
   } else if (tid == 32) {
     // the descriptors of the first copies
-    const CUtensorMap* maps[7] = {&tm.wg32, &tm.wu32, &tm.wg, &tm.wu, &tm.x, &tm.sg32, &tm.su32};
+    const CUtensorMap* maps[6] = {&tm.gu32, &tm.gu, &tm.x32, &tm.x, &tm.sgu32, &tm.sgu};
 #pragma unroll
-    for (int i = 0; i < 7; ++i) ptx::prefetch_tensormap(maps[i]);
+    for (int i = 0; i < 6; ++i) ptx::prefetch_tensormap(maps[i]);
   }
   if (warp == 1) {
     ptx::tmem_alloc(s_tmem, p.tmem_cols);
@@ -211,37 +228,29 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       // poll every block's words until all are nonzero; a nonzero word is complete (one
       // 32-bit store), so its ids go into the shared mask as it is seen (or-ing twice is
       // harmless)
-      const int nw = spec_words(p.k), total = p.spec_blocks * nw;
+      const int nw = kMask ? kSpecMaskWords : spec_words(p.k), total = p.spec_blocks * nw;
       if (lane < kMaxExperts / 32) s_mask[lane] = 0u;
       __syncwarp();
       bool bad = false;
       const uint64_t t0 = ptx::globaltimer_ns();
       for (;;) {
         bool all = true;
-        if (kMask) {
-          // masks: a block's words are read once its marker (stored last, with release
-          // semantics) is seen by an acquire load; or-ing a mask twice is harmless
-          for (int b = lane; b < p.spec_blocks; b += 32) {
-            const uint32_t* wb = p.spec_words + (size_t)b * kSpecMaskWords;
-            if (ld_acquire(reinterpret_cast<const int32_t*>(wb + kMaxExperts / 32)) == 0) {
-              all = false;
-              continue;
-            }
-#pragma unroll
-            for (int w = 0; w < kMaxExperts / 32; ++w) {
-              const uint32_t m = ld_relaxed_u32(wb + w);
-              if (m != 0u) {
-                if (32 * w >= p.E || (32 * w + 31 >= p.E && (m >> (p.E - 32 * w)) != 0u))
-                  bad = true;
-                atomicOr(&s_mask[w], m);
-              }
-            }
-          }
-        } else
         for (int i = lane; i < total; i += 32) {
           const uint32_t w = ld_relaxed_u32(p.spec_words + i);
           if (w == 0u) {
             all = false;
+            continue;
+          }
+          if (kMask) {
+            // member bits of experts e0 .. e0 + 23 (or-ing a mask twice is harmless)
+            const int e0 = 24 * (i % nw), q = e0 >> 5, sh = e0 & 31;
+            const uint32_t m = w & 0xffffffu;
+            if (e0 + 24 > p.E && (e0 >= p.E ? m : m >> (p.E - e0)) != 0u) {
+              bad = true;
+              continue;
+            }
+            if (m << sh) atomicOr(&s_mask[q], m << sh);
+            if (sh > 8 && (m >> (32 - sh)) != 0u) atomicOr(&s_mask[q + 1], m >> (32 - sh));
             continue;
           }
           const int r0 = 3 * (i % nw);
@@ -294,8 +303,6 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
           const bool sh = b < ngse;
           const int m = sh ? b : (b - ngse) % ngre;
           const int e = sh ? 0 : (int)s_spec[(b - ngse) / ngre];
-          const CUtensorMap* mg = h32e ? (sh ? &tm.sg32 : &tm.wg32) : (sh ? &tm.sg : &tm.wg);
-          const CUtensorMap* mu = h32e ? (sh ? &tm.su32 : &tm.wu32) : (sh ? &tm.su : &tm.wu);
           const int arow = (sh ? 0 : e * pI) + m * hge;
           const uint64_t pw = ptx::policy_evict_first(), px = ptx::policy_evict_last();
           early = Se < kce ? Se : kce;
@@ -303,14 +310,8 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
           for (int c = 0; c < early; ++c) {
             ptx::mbar_arrive_expect_tx(&full[c], kAStage + kbge * bbox);
             uint8_t* a_dst = smem + c * slote;
-            uint8_t* b_dst = a_dst + kAStage;
-            for (int kb = 0; kb < kbge; ++kb) {
-              const int kx = (c * kbge + kb) * kTileK;
-              ptx::tma_load_2d(a_dst + kb * 2 * hge * 128, mg, &full[c], kx, arow, pw);
-              ptx::tma_load_2d(a_dst + kb * 2 * hge * 128 + hge * 128, mu, &full[c], kx, arow,
-                               pw);
-              ptx::tma_load_2d(b_dst + kb * bbox, &tm.x, &full[c], kx, 0, px);
-            }
+            load_gate_up(tm, p, a_dst, &full[c], sh, h32e, arow, c * kbge, pw);
+            ptx::tma_load_3d(a_dst + kAStage, h32e ? &tm.x32 : &tm.x, &full[c], 0, 0, c * kbge, px);
           }
         }
       }
@@ -455,10 +456,6 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       int gi, m;
       gu_unit(u, gi, m);
       const Grp g = group_w(gi);
-      const CUtensorMap* mg =
-          hg == 32 ? (g.shared ? &tm.sg32 : &tm.wg32) : (g.shared ? &tm.sg : &tm.wg);
-      const CUtensorMap* mu =
-          hg == 32 ? (g.shared ? &tm.su32 : &tm.wu32) : (g.shared ? &tm.su : &tm.wu);
       const int arow = (g.shared ? 0 : g.e * p.I) + m * hg;
       if (first) ED_SET(10, u);
       for (int c = first ? early : 0; c < kc; ++c) {
@@ -466,14 +463,8 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
         if (first && c == 0) ED_AT(28);
         if (first && c == kc - 1) ED_AT(29);
         ptx::mbar_arrive_expect_tx(&full[stage], kAStage + kbg * bbox);
-        uint8_t* a_dst = slot_a(stage);
-        uint8_t* b_dst = slot_b(stage);
-        for (int kb = 0; kb < kbg; ++kb) {
-          const int kx = (c * kbg + kb) * kTileK;
-          ptx::tma_load_2d(a_dst + kb * abox_g, mg, &full[stage], kx, arow, pol_w);
-          ptx::tma_load_2d(a_dst + kb * abox_g + hg * 128, mu, &full[stage], kx, arow, pol_w);
-          ptx::tma_load_2d(b_dst + kb * bbox, &tm.x, &full[stage], kx, 0, pol_x);
-        }
+        load_gate_up(tm, p, slot_a(stage), &full[stage], g.shared, h32, arow, c * kbg, pol_w);
+        ptx::tma_load_3d(slot_b(stage), h32 ? &tm.x32 : &tm.x, &full[stage], 0, 0, c * kbg, pol_x);
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -494,11 +485,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       for (int c = 0; c < pre; ++c, ++done) {
         if (!wait(&empty[stage], phase ^ 1u, v)) { ok = false; break; }
         ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
-        uint8_t* a_dst = slot_a(stage);
-#pragma unroll
-        for (int kb = 0; kb < kKB; ++kb)
-          ptx::tma_load_2d(a_dst + kb * kABox, md, &full[stage], c * kStageK + kb * kTileK, arow,
-                           pol_w);
+        ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -523,11 +510,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
         int st = st0;
         for (int c = 0; c < done; ++c) {
           if (ok) {
-            uint8_t* b_dst = slot_b(st);
-#pragma unroll
-            for (int kb = 0; kb < kKB; ++kb)
-              ptx::tma_load_2d(b_dst + kb * bbox, &tm.h, &full[st], c * kStageK + kb * kTileK,
-                               gi * p.n_pad, pol_x);
+            ptx::tma_load_3d(slot_b(st), &tm.h, &full[st], 0, gi * p.n_pad, c * kKB, pol_x);
           } else {
             // keep the barrier accounting whole: complete the stage without B data
             ptx::mbar_complete_tx_local(&full[st], bstage);
@@ -538,14 +521,8 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       for (int c = pre; c < ndk && ok; ++c) {
         if (!wait(&empty[stage], phase ^ 1u, v)) { ok = false; break; }
         ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
-        uint8_t* a_dst = slot_a(stage);
-        uint8_t* b_dst = slot_b(stage);
-#pragma unroll
-        for (int kb = 0; kb < kKB; ++kb) {
-          const int kx = c * kStageK + kb * kTileK;
-          ptx::tma_load_2d(a_dst + kb * kABox, md, &full[stage], kx, arow, pol_w);
-          ptx::tma_load_2d(b_dst + kb * bbox, &tm.h, &full[stage], kx, gi * p.n_pad, pol_x);
-        }
+        ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
+        ptx::tma_load_3d(slot_b(stage), &tm.h, &full[stage], 0, gi * p.n_pad, c * kKB, pol_x);
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -627,13 +604,11 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     const int et = tid - 64;                      // 0..127
     const int row = q * 32 + lane;                // accumulator row of this thread
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    const bool is_gate = q < 2;
     // gate/up accumulator (M = 2 hg): row r sits in TMEM lane r for M = 128 and in lane
-    // 32 (r / 16) + r % 16 for M = 64, so each quadrant holds rq = hg / 2 rows in its first
-    // rq lanes: gate rows in quadrants 0-1, the matching up rows in quadrants 2-3
-    const int rq = hg / 2;
-    const bool g_act = lane < rq;
-    const int rr = (q & 1) * rq + lane;           // row within the hg-row slice
+    // 32 (r / 16) + r % 16 for M = 64. The A tile holds 8 gate rows and the same 8 up rows in
+    // turn, so the up row of a gate lane l is in lane l + 8 of the same warp
+    const bool g_act = hg == 64 || lane < 16;
+    const int rr = (hg == 64 ? 16 * q + 8 * (lane >> 4) : 8 * q) + (lane & 7);   // row of the tile
     const int n_mma = (p.T + 15) & ~15;
     const uint32_t part1 = (uint32_t)(p.n_acc * p.n_pad);   // column offset of part 1
     // 16 columns of an accumulator: the sum of its two parts
@@ -660,45 +635,30 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       ptx::tc_fence_after();
       const uint32_t tbase = tmem_base + lane_off + (uint32_t)(acc * p.n_pad);
       // the H tile (n_pad token rows x hg columns, bf16) is laid out in the staging tile as
-      // hg / 32 row-major boxes of 32 columns, then stored by TMA
-      uint8_t* hbox = reinterpret_cast<uint8_t*>(stage_t);
-      // per 16-token slice: every row's 16 values go to the exchange tile (gate rows
-      // 0..hg-1, up rows hg..2hg-1), then all 128 threads take hg / 8 adjacent columns of one
-      // token each (loads first, then the SwiGLU, then one 8- or 16-byte store)
-      const int cpt = hg >> 3, xc = et >> 3, col0 = (et & 7) * cpt;
-      uint8_t* hdst = hbox + (col0 >> 5) * p.n_pad * 64 + (col0 & 31) * 2;
+      // hg / 32 row-major boxes of 32 columns, then stored by TMA. Per 16-token slice a gate lane
+      // gives its last 8 columns to the lane that holds its row's up values and takes that
+      // one's first 8; each then has gate and up of one row for 8 tokens
+      const bool gate_first = (gi < p.has_shared ? p.sgu_box : p.gu_box) != 2;
+      const bool is_gate = ((lane & 8) == 0) == gate_first;
+      uint8_t* hdst = hbox + (rr >> 5) * p.n_pad * 64 + (rr & 30) * 2;
       for (int c0 = 0; c0 < n_mma; c0 += 16) {
         float v[16];
         acc_ld16(tbase + c0, v);
         if (first && et == 0 && c0 == 0) ED_AT(23);
-        if (g_act) {
-          float* xr = xchg + ((is_gate ? 0 : hg) + rr) * kXStride;
+        float h[8];
 #pragma unroll
-          for (int c = 0; c < 16; ++c) xr[c] = v[c];
+        for (int j = 0; j < 8; ++j) {
+          const float other =
+              __shfl_xor_sync(0xffffffffu, is_gate ? v[8 + j] : v[j], kGateRows);
+          h[j] = silu_f(is_gate ? v[j] : other) * (is_gate ? other : v[8 + j]);
         }
-        named_bar_sync(2, 128);
-        if (first && et == 0 && c0 == 0) ED_AT(24);
-        float gv[8], uv[8];
+        uint32_t w[4];
+        ptx::pair_rows(h, w);
+        if (g_act) {
+          uint8_t* hrow = hdst + (c0 + (is_gate ? 0 : 8) + 4 * (lane & 1)) * 64;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (j < cpt) {
-            gv[j] = xchg[(col0 + j) * kXStride + xc];
-            uv[j] = xchg[(hg + col0 + j) * kXStride + xc];
-          }
-        uint32_t hp[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (2 * j < cpt) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(silu_f(gv[2 * j]) * uv[2 * j],
-                                                            silu_f(gv[2 * j + 1]) * uv[2 * j + 1]);
-            hp[j] = *reinterpret_cast<const uint32_t*>(&h2);
-          }
-        uint8_t* hrow = hdst + (c0 + xc) * 64;
-        if (cpt == 4)
-          *reinterpret_cast<uint2*>(hrow) = make_uint2(hp[0], hp[1]);
-        else
-          *reinterpret_cast<uint4*>(hrow) = make_uint4(hp[0], hp[1], hp[2], hp[3]);
-        named_bar_sync(2, 128);   // the exchange tile is rewritten by the next slice
+          for (int j = 0; j < 4; ++j) *reinterpret_cast<uint32_t*>(hrow + j * 64) = w[j];
+        }
       }
       if (first && et == 0) ED_AT(25);
       ptx::tc_fence_before();
@@ -745,57 +705,39 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     for (int v = v0; v < ND; v += nb) {
       const int gi = v / ndn, i = v % ndn;
       const Grp g = group(gi);
-      if (!g.shared && et < g.n) tok[et] = __ldcg(p.rows + g.row0 + et) / p.k;
-      const bool ok = epi_all(wait(&acc_full[acc], acc_phase, v));   // also orders tok[]
+      // the output row of every token's column: its place in the dispatch, or the token's own
+      // (shared expert)
+      if (et < kMaxTok) s_row[et] = g.shared && et < p.T ? et : -1;
+      if (!g.shared) {
+        named_bar_sync(2, 128);
+        if (et < g.n) {
+          const int t = __ldcg(p.rows + g.row0 + et) / p.k;
+          if (t >= 0 && t < p.T) s_row[t] = g.row0 + et;
+        }
+      }
+      const bool ok = epi_all(wait(&acc_full[acc], acc_phase, v));   // also orders s_row[]
       if (!ok) break;
       if (first && et == 0) ED_AT(14);
       ptx::tc_fence_after();
       const uint32_t tbase = tmem_base + lane_off + (uint32_t)(acc * p.n_pad);
-      // the accumulator column of token t is the group's output for t: the tile goes through
-      // shared memory as [token][128 rows] fp32, then one 512-B bulk copy per kept row (every
-      // token for the shared expert, the routed ones in dispatch order otherwise)
-      float* stg = stage_t;
+      // the accumulator column of token t is the group's output for t; a warp's 32 rows of one
+      // token are 128 bytes of its output row, stored straight from the registers (through
+      // shared memory and one bulk copy per row this took 0.8 us at 15 rows, 1.9 at 30)
+      float* dst = (g.shared ? p.yshared : p.yslot) + (size_t)i * kTileM + row;
       for (int c0 = 0; c0 < n_mma; c0 += 16) {
         float vv[16];
         acc_ld16(tbase + c0, vv);
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
-          if (c0 + c < p.T) stg[(c0 + c) * kTileM + row] = vv[c];
+        for (int c = 0; c < 16; ++c) {
+          const int r = s_row[c0 + c];
+          if (r >= 0) __stcg(dst + (size_t)r * p.d, vv[c]);
+        }
       }
+      if (first && et == 0) ED_AT(15);
       ptx::tc_fence_before();
       ptx::mbar_arrive(&acc_empty[acc]);
       if (++acc == p.n_acc) { acc = 0; acc_phase ^= 1u; }
-      if (first && et == 0) ED_AT(15);
-      ptx::fence_proxy_async_smem();
-      named_bar_sync(2, 128);
-      if (et < 32) {
-        if (first && et == 0) ED_AT(16);
-        const int nrows = g.shared ? p.T : g.n;
-        // every token kept (the shared expert; a routed group that all T tokens use, whose
-        // dispatch rows are then tokens 0..T-1 in order): the staging tile is the rows' image,
-        // stored 8 rows per tensor copy; otherwise one 512-B row copy per lane
-        bool dense = nrows == p.T && (p.T & 7) == 0;
-        if (dense && !g.shared)
-          for (int r = et; r < nrows; r += 32) dense = dense && tok[r] == r;
-        dense = __all_sync(0xffffffffu, dense);
-        if (dense) {
-          if (et == 0)
-            for (int r8 = 0; r8 < nrows; r8 += 8)
-              tma_store_2d(g.shared ? &tm.ysh : &tm.ys, stg + r8 * kTileM, i * kTileM,
-                           (g.shared ? 0 : g.row0) + r8);
-        } else {
-          const size_t col = (size_t)i * kTileM;
-          for (int r = et; r < nrows; r += 32) {
-            const int t = g.shared ? r : tok[r];
-            float* dst = g.shared ? p.yshared + (size_t)r * p.d + col
-                                  : p.yslot + (size_t)(g.row0 + r) * p.d + col;
-            if (t >= 0 && t < p.T) bulk_store(dst, stg + t * kTileM, kTileM * 4);
-          }
-        }
-        if (first && et == 0) ED_AT(17);
-        bulk_commit_wait_read();   // the staging tile is rewritten by the next unit
-      }
-      named_bar_sync(2, 128);   // tok[] and the staging tile are rewritten by the next unit
+      named_bar_sync(2, 128);   // s_row[] is rewritten by the next unit
       if (first && et == 0) ED_AT(8);
       first = false;
     }
@@ -835,33 +777,53 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// bf16 matrix [rows, cols] row-major, box = 64 columns (128 B) x box_rows rows with the
-// 128-B swizzle, or (plain) box_cols columns x box_rows rows without swizzle.
+// bf16 matrix [rows, cols] row-major as [cols / 64][rows][64]: a box of box_rows rows and
+// `ksteps` 64-column steps, 128-B swizzle.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
-              bool plain = false, uint32_t box_cols = 64) {
+              uint32_t ksteps) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  const cuuint64_t dims[3] = {64, rows, cols / 64};
+  const cuuint64_t strides[2] = {cols * 2, 128};
+  const cuuint32_t box[3] = {64, box_rows, ksteps};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Two such matrices of one shape, the one at the lower address first, 8 rows of each in turn: a
+// box of `hg` rows of each and `ksteps` steps. Their distance is a stride of the map: a
+// multiple of 16 bytes below 2^40. Returns 1 (a first), 2 (b first) or 0: no such map.
+int make_map_two(CUtensorMap* m, const void* a, const void* b, uint64_t rows, uint64_t cols,
+                 uint32_t hg, uint32_t ksteps) {
+  EncodeTiledFn enc = encode_fn();
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  const uint64_t dist = pa < pb ? pb - pa : pa - pb;
+  if (enc == nullptr || dist == 0 || dist % 16 != 0 || dist >= ((uint64_t)1 << 40)) return 0;
+  const cuuint64_t dims[5] = {64, kGateRows, 2, rows / kGateRows, cols / 64};
+  const cuuint64_t strides[4] = {cols * 2, dist, cols * 2 * kGateRows, 128};
+  const cuuint32_t box[5] = {64, kGateRows, 2, hg / kGateRows, ksteps};
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  if (enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pa < pb ? a : b), dims, strides,
+          box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return 0;
+  return pa < pb ? 1 : 2;
+}
+
+// bf16 matrix [rows, cols] row-major, box = 32 columns x box_rows rows, no swizzle.
+bool make_map_plain(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols,
+                    uint32_t box_rows) {
   EncodeTiledFn enc = encode_fn();
   if (enc == nullptr) return false;
   const cuuint64_t dims[2] = {cols, rows};
   const cuuint64_t strides[1] = {cols * 2};
-  const cuuint32_t box[2] = {plain ? box_cols : 64u, box_rows};
+  const cuuint32_t box[2] = {32, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-             estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             plain ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// fp32 matrix [rows, cols] row-major, box = 128 columns x 8 rows, no swizzle.
-bool make_map_f32(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
-  EncodeTiledFn enc = encode_fn();
-  if (enc == nullptr) return false;
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {cols * 4};
-  const cuuint32_t box[2] = {(cuuint32_t)kTileM, 8};
-  const cuuint32_t estr[2] = {1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box,
              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // Opt-in shared memory per CTA; without a device (host-side planning) the sm_100-family
@@ -883,9 +845,9 @@ uint32_t pow2_cols(uint32_t n) {
   return c;
 }
 
-// Shared memory besides the ring: staging tile, SwiGLU exchange, token list, barriers.
+// Shared memory besides the ring: staged H box, row list, barriers.
 size_t fixed_smem(int n_pad) {
-  return 1024 /* alignment */ + (size_t)kTileM * (n_pad + 1) * 4 + kXchgBytes + kMaxTok * 4 +
+  return 1024 /* alignment */ + (size_t)2 * 64 * n_pad + kMaxTok * 4 +
          (size_t)(2 * kMaxStagesD + 9) * 8 + 16 + kMaxExperts + kMaxExperts / 8 + 48;
 }
 
@@ -932,29 +894,34 @@ cudaError_t launch_experts_decode(const ExpertArgs& a, cudaStream_t s) {
   const int n_pad = ((a.T + 15) / 16) * 16;
   const int imax = a.I > a.Is ? a.I : a.Is;
 
-  DMaps m;
-  bool ok = make_map(&m.wg, a.w_gate, (uint64_t)a.E * a.I, a.d, 64) &&
-            make_map(&m.wu, a.w_up, (uint64_t)a.E * a.I, a.d, 64) &&
-            make_map(&m.wg32, a.w_gate, (uint64_t)a.E * a.I, a.d, 32) &&
-            make_map(&m.wu32, a.w_up, (uint64_t)a.E * a.I, a.d, 32) &&
-            make_map(&m.wd, a.w_down, (uint64_t)a.E * a.d, a.I, kTileM) &&
-            make_map(&m.x, a.x, (uint64_t)a.T, a.d, (uint32_t)n_pad) &&
-            make_map(&m.h, a.hdense, (uint64_t)(a.E + 1) * n_pad, (uint64_t)imax,
-                     (uint32_t)n_pad) &&
-            make_map(&m.hst, a.hdense, (uint64_t)(a.E + 1) * n_pad, (uint64_t)imax,
-                     (uint32_t)n_pad, true, 32) &&
-            make_map_f32(&m.ys, a.yslot, (uint64_t)a.T * a.k, a.d) &&
-            make_map_f32(&m.ysh, a.yshared, (uint64_t)a.T, a.d);
-  if (ok && has_shared)
-    ok = make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, 64) &&
-         make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, 64) &&
-         make_map(&m.sg32, a.ws_gate, (uint64_t)a.Is, a.d, 32) &&
-         make_map(&m.su32, a.ws_up, (uint64_t)a.Is, a.d, 32) &&
-         make_map(&m.sd, a.ws_down, (uint64_t)a.d, a.Is, kTileM);
-  if (!has_shared) { m.sg = m.wg; m.su = m.wu; m.sd = m.wd; m.sg32 = m.wg32; m.su32 = m.wu32; }
+  // (only the maps that this call uses: each costs the host time)
+  DMaps m{};
+  DParams p{};
+  const uint64_t gu_rows = (uint64_t)a.E * a.I, h_rows = (uint64_t)(a.E + 1) * n_pad;
+  bool ok = make_map(&m.wd, a.w_down, (uint64_t)a.E * a.d, a.I, kTileM, kKB) &&
+            make_map(&m.x, a.x, (uint64_t)a.T, a.d, (uint32_t)n_pad, kTileM / 64) &&
+            make_map(&m.h, a.hdense, h_rows, (uint64_t)imax, (uint32_t)n_pad, kKB) &&
+            make_map_plain(&m.hst, a.hdense, h_rows, (uint64_t)imax, (uint32_t)n_pad);
+  p.gu_box = make_map_two(&m.gu, a.w_gate, a.w_up, gu_rows, a.d, 64, kTileM / 64);
+  if (ring.h32_ok) {
+    ok = ok && make_map(&m.x32, a.x, (uint64_t)a.T, a.d, (uint32_t)n_pad, kTileM / 32);
+    if (p.gu_box != 0)
+      p.gu_box = make_map_two(&m.gu32, a.w_gate, a.w_up, gu_rows, a.d, 32, kTileM / 32);
+  }
+  if (p.gu_box == 0)
+    ok = ok && make_map(&m.wg, a.w_gate, gu_rows, a.d, kGateRows, 1) &&
+         make_map(&m.wu, a.w_up, gu_rows, a.d, kGateRows, 1);
+  if (has_shared) {
+    ok = ok && make_map(&m.sd, a.ws_down, (uint64_t)a.d, a.Is, kTileM, kKB);
+    p.sgu_box = make_map_two(&m.sgu, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d, 64, kTileM / 64);
+    if (ring.h32_ok && p.sgu_box != 0)
+      p.sgu_box = make_map_two(&m.sgu32, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d, 32, kTileM / 32);
+    if (p.sgu_box == 0)
+      ok = ok && make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, kGateRows, 1) &&
+           make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, kGateRows, 1);
+  }
   if (!ok) return cudaErrorInvalidValue;
 
-  DParams p{};
   p.n_unique = a.n_unique;
   p.unique_ids = a.unique_ids;
   p.offsets = a.offsets;

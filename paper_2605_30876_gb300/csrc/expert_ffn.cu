@@ -118,6 +118,7 @@ struct Maps {
 using ptx::fence_proxy_async_global;
 using ptx::ld_acquire;
 using ptx::named_bar_sync;
+using ptx::pair_rows;
 using ptx::red_release_add;
 
 // silu with the fast divide: H is rounded to bf16 right after
@@ -127,28 +128,6 @@ __device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __
 // after this launch, while the weights stream through L2 with evict-first)
 __device__ __forceinline__ void st_u32_keep(void* p, uint32_t v, uint64_t pol) {
   asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
-}
-
-// A thread holds eight tokens' values of one row; the row of lane xor 1 is its neighbour. After
-// the swap it holds two neighbouring rows (the lower one first) of four tokens: the even
-// lane tokens 0-3, the odd lane tokens 4-7, one bf16 pair per token, so that a warp's stores
-// are 4-byte words of 64-byte runs (half the stores of single bf16 values).
-__device__ __forceinline__ void pair_rows(const float (&v)[8], uint32_t (&w)[4]) {
-  uint32_t pk[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    pk[i] = *reinterpret_cast<const uint32_t*>(&b);
-  }
-  const bool odd = threadIdx.x & 1;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const uint32_t mine = odd ? pk[2 + i] : pk[i];
-    const uint32_t other = __shfl_xor_sync(0xffffffffu, odd ? pk[i] : pk[2 + i], 1);
-    const uint32_t lo = odd ? other : mine, hi = odd ? mine : other;
-    w[2 * i] = __byte_perm(lo, hi, 0x5410);
-    w[2 * i + 1] = __byte_perm(lo, hi, 0x7632);
-  }
 }
 
 // AND of `v` over the kEpiThreads epilogue threads (named barrier 1), so that they take the

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace dmoe {
@@ -105,6 +106,24 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                            int32_t x, int32_t y, int32_t z, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(x), "r"(y), "r"(z), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                            int32_t x, int32_t y, int32_t z, int32_t w, int32_t v,
+                                            uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(x), "r"(y), "r"(z), "r"(w),
+      "r"(v), "l"(policy)
+      : "memory");
+}
 // The same by a CTA of a pair: into its own shared memory, the bytes signalled on a barrier of
 // either CTA of the pair (a shared::cluster address).
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map,
@@ -379,6 +398,27 @@ __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N) {
 }
 
 // ------------------------------------------------------------------ epilogue helpers
+// A thread holds eight tokens' values of one row; the row of lane xor 1 is its neighbour. After
+// the swap it holds two neighbouring rows (the lower one first) of four tokens: the even
+// lane tokens 0-3, the odd lane tokens 4-7, one bf16 pair per token, so that a warp's stores
+// are 4-byte words of 64-byte runs (half the stores of single bf16 values).
+__device__ __forceinline__ void pair_rows(const float (&v)[8], uint32_t (&w)[4]) {
+  uint32_t pk[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    pk[i] = *reinterpret_cast<const uint32_t*>(&b);
+  }
+  const bool odd = threadIdx.x & 1;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t mine = odd ? pk[2 + i] : pk[i];
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, odd ? pk[i] : pk[2 + i], 1);
+    const uint32_t lo = odd ? other : mine, hi = odd ? mine : other;
+    w[2 * i] = __byte_perm(lo, hi, 0x5410);
+    w[2 * i + 1] = __byte_perm(lo, hi, 0x7632);
+  }
+}
 __device__ __forceinline__ void named_bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }

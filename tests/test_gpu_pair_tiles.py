@@ -1,7 +1,9 @@
-"""The general expert launch (more than 64 tokens) where its tiles can go wrong, against the CPU
-oracle: tiles of 32 to 256 token rows with remainders, blocks that fill half tiles in twos or
+"""The expert launches where their tiles can go wrong, against the CPU oracle. The general one (more
+than 64 tokens): tiles of 32 to 256 token rows with remainders, blocks that fill half tiles in twos or
 fours, blocks that fill none, d and I of an odd number of 128-row tiles, more token tiles than
-one, fewer units than clusters, and gate and up weights that no single copy can bring."""
+one, fewer units than clusters, and gate and up weights that no single copy can bring. The
+decode-size one: both unit heights, the smallest and the largest token count, outputs kept by
+few tokens, and the same two forms of the weights' copies."""
 import numpy as np
 import pytest
 import torch
@@ -32,11 +34,19 @@ CASES = {
                                  top_k=8),
     "token_300_d384_I384": SMALL.with_(block_size=60, n_blocks=5, mode=ROUTE_TOKEN, n_experts=8,
                                        top_k=8, d_model=384, d_ff=384, d_ff_shared=256),
+    # decode size: 32-row gate/up units (few experts) and 64-row ones, 1 to 64 tokens
+    "decode_1": SMALL.with_(block_size=1, n_blocks=1),
+    "decode_5x12": SMALL.with_(block_size=12, n_blocks=5),
+    "decode_64_all": SMALL.with_(block_size=64, n_blocks=1, n_experts=8, top_k=8, d_model=512),
+    "decode_token_61": SMALL.with_(block_size=61, n_blocks=1, mode=ROUTE_TOKEN, n_experts=256,
+                                   top_k=16, d_ff=256, d_ff_shared=512),
+    "decode_d384_p06": SMALL.with_(block_size=17, n_blocks=3, top_p=0.6, d_model=384),
 }
 
 
 @pytest.mark.parametrize("name,one_tensor", [(n, False) for n in CASES] +
-                         [("blocks_24x5", True), ("token_300_d384_I384", True)])
+                         [(n, True) for n in ("blocks_24x5", "token_300_d384_I384",
+                                               "decode_5x12", "decode_token_61")])
 def test_layer_matches_oracle(name, one_tensor):
     shape = CASES[name]
     m = P.dm()
