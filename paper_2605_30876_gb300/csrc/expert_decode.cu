@@ -724,13 +724,21 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       // token are 128 bytes of its output row, stored straight from the registers (through
       // shared memory and one bulk copy per row this took 0.8 us at 15 rows, 1.9 at 30)
       float* dst = (g.shared ? p.yshared : p.yslot) + (size_t)i * kTileM + row;
-      for (int c0 = 0; c0 < n_mma; c0 += 16) {
-        float vv[16];
-        acc_ld16(tbase + c0, vv);
+      // (eight columns at a time: this code runs a few times per launch, so its size costs more
+      // than the shorter TMEM loads)
+#pragma unroll 1
+      for (int c0 = 0; c0 < n_mma; c0 += 8) {
+        float va[8], vb[8];
+        ptx::tmem_ld8(tbase + c0, va);
+        ptx::tmem_ld8(tbase + c0 + part1, vb);
+        const int4 r0 = *reinterpret_cast<const int4*>(s_row + c0);
+        const int4 r1 = *reinterpret_cast<const int4*>(s_row + c0 + 4);
+        const int r[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+        ptx::tmem_ld_wait();
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int r = s_row[c0 + c];
-          if (r >= 0) __stcg(dst + (size_t)r * p.d, vv[c]);
+        for (int c = 0; c < 8; ++c) {
+          asm volatile("" : "+f"(va[c]), "+f"(vb[c]));   // the values exist only after the wait
+          if (r[c] >= 0) __stcg(dst + (size_t)r[c] * p.d, va[c] + vb[c]);
         }
       }
       if (first && et == 0) ED_AT(15);
