@@ -16,7 +16,7 @@
 //                             e holds expert e's weights over d), the MMA's B operand
 //   router_logits_tc_kernel   one CTA per (128 tokens, slice of d, group of N experts; N =
 //                             E / nsplit, a multiple of 32, at most 256), no cross-CTA step:
-//     warp 0     TMA, two stages: x chunk (128 tokens x 64 of d, 128-B swizzle, rows past
+//     warp 0     TMA, up to four stages, one per chunk where they fit: x chunk (128 tokens x 64 of d, 128-B swizzle, rows past
 //                T read as zero) and the three parts' chunks (N rows x 64)
 //     warp 1     TMEM allocation; lane 0 issues D[128 x N] += x * part^T, 4 K-steps of 16
 //                per chunk and part (hi into one accumulator, mid and lo into the other)
@@ -25,6 +25,8 @@
 //                experts x 128 tokens with the 128-B swizzle, which thread 0 then stores by
 //                TMA (rows past T are not written)
 // Every mbarrier wait is bounded (1 s): a timeout is recorded and the CTA unwinds.
+#include <algorithm>
+
 #include "dmoe_internal.cuh"
 #include "sm100_ptx.cuh"
 #include "trace_log.cuh"
@@ -47,6 +49,7 @@ namespace {
 constexpr int kLtM = 128;                     // tokens per tile (MMA M)
 constexpr int kLtKC = 64;                     // d per chunk: one 128-B row of bf16
 constexpr int kLtMaxDS = 256;                 // d per CTA at most (16 hi MMAs)
+constexpr int kLtStages = kLtMaxDS / kLtKC;    // stages at most: one per chunk of the slice
 constexpr int kLtThreads = 128;
 constexpr int kLtXBytes = kLtM * 128;         // 16 KB
 constexpr uint64_t kLtTimeoutNs = 1000000000ull;
@@ -59,6 +62,7 @@ struct LtArgs {
   L2Prefetch shared_pf;
   int T, d, E, ds;    // ds: d per slice (blockIdx.y)
   int N;              // experts per CTA (blockIdx.z: experts N z .. N z + N - 1)
+  int stages;         // chunks in flight (lt_stages)
 };
 
 // parts[p][e][i] for the tile of 32 experts x 64 of d: thread (e, 8-wide run of d) reads
@@ -111,7 +115,7 @@ __global__ void __launch_bounds__(kLtThreads, 1)
 router_logits_tc_kernel(const __grid_constant__ LtArgs f) {
   extern __shared__ uint8_t lt_raw[];
   uint8_t* smem = lt_raw + ((1024u - (ptx::smem_addr(lt_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t full[2], empty[2], acc_full;
+  __shared__ __align__(8) uint64_t full[kLtStages], empty[kLtStages], acc_full;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -133,17 +137,13 @@ router_logits_tc_kernel(const __grid_constant__ LtArgs f) {
   if (tid == 0) {
     ptx::prefetch_tensormap(&f.xmap);
     ptx::prefetch_tensormap(&f.pmap);
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < f.stages; ++s) {
       ptx::mbar_init(&full[s], 1);
       ptx::mbar_init(&empty[s], 1);
     }
     ptx::mbar_init(&acc_full, 1);
     ptx::fence_mbarrier_init();
     s_abort = 0;
-    // the shared expert's weights are pulled into L2 for the expert launch
-    issue_shared_prefetch(f.shared_pf,
-                          (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x),
-                          (int)(gridDim.x * gridDim.y * gridDim.z));
   }
   if (warp == 1) {
     ptx::tmem_alloc(&s_tmem, t_cols);
@@ -171,9 +171,9 @@ router_logits_tc_kernel(const __grid_constant__ LtArgs f) {
       // ================= TMA producer
       const uint64_t pol = ptx::policy_evict_last();   // x and the parts are re-read by tiles
       for (int c = 0; c < nch; ++c) {
-        const int s = c & 1;
-        const uint32_t ph = (uint32_t)((c >> 1) & 1);
-        if (c >= 2 && !wait(&empty[s], ph ^ 1u, 100 + c)) break;
+        const int s = c % f.stages;
+        const uint32_t ph = (uint32_t)((c / f.stages) & 1);
+        if (c >= f.stages && !wait(&empty[s], ph ^ 1u, 100 + c)) break;
         ptx::mbar_arrive_expect_tx(&full[s], (uint32_t)slot);
         const int k0 = k_base + c * kLtKC;
         ptx::tma_load_2d(x_buf(s), &f.xmap, &full[s], k0, m0, pol);
@@ -182,14 +182,19 @@ router_logits_tc_kernel(const __grid_constant__ LtArgs f) {
           ptx::tma_load_2d(p_buf(s, part), &f.pmap, &full[s], k0, part * E + e_base, pol);
       }
       RTC_AT(2);
+      // the shared expert's weights are pulled into L2 for the expert launch; behind this CTA's
+      // own loads, which the copy engine would otherwise serve after them
+      issue_shared_prefetch(f.shared_pf,
+                            (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x),
+                            (int)(gridDim.x * gridDim.y * gridDim.z));
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // ================= MMA issuer
       const uint32_t idesc = ptx::idesc_bf16(kLtM, (uint32_t)N);
       for (int c = 0; c < nch; ++c) {
-        const int s = c & 1;
-        const uint32_t ph = (uint32_t)((c >> 1) & 1);
+        const int s = c % f.stages;
+        const uint32_t ph = (uint32_t)((c / f.stages) & 1);
         if (!wait(&full[s], ph, 300 + c)) break;
         if (c == 0) RTC_AT(3);
         ptx::tc_fence_after();
@@ -287,7 +292,23 @@ bool encode_bf16_2d(EncodeFn enc, CUtensorMap* m, const void* base, uint64_t row
          CUDA_SUCCESS;
 }
 
-size_t lt_smem_bytes(int E) { return 2 * ((size_t)kLtXBytes + 3 * (size_t)E * 128) + 1024; }
+constexpr int kLtSmemMax = 226 * 1024;   // dynamic: the barriers are static shared memory
+
+// As many stages as the slice has chunks and shared memory holds (4 up to N = 64, 3 at 128, 2
+// at 256); at least two, which the epilogue's boxes need (16 KB per 32 experts). The launch is
+// latency: at T = 256, d = 2048, E = 128 (128 CTAs of 4 chunks) the first chunk landed 0.6 us
+// after entry and, with two stages, the last was asked for at 1.9 us, once the MMAs had given
+// the first back. All four at once, and the shared expert's L2 prefetch behind them instead of
+// before, took the layer of 256 tokens (top-k blocks) from 49.95 to 48.4 us and that of 300
+// from 67.1 to 66.1; at T = 2048 (three stages) it is the same to 0.3 %.
+int lt_stages(int N, int nch) {
+  const int fit = (kLtSmemMax - 1024) / (kLtXBytes + 3 * N * 128);
+  return std::max(2, std::min(std::min(nch, kLtStages), fit));
+}
+
+size_t lt_smem_bytes(int N, int stages) {
+  return stages * ((size_t)kLtXBytes + 3 * (size_t)N * 128) + 1024;
+}
 
 bool encode_part_3d(EncodeFn enc, CUtensorMap* m, float* base, int S, int T, int E) {
   const cuuint64_t dims[3] = {(cuuint64_t)E, (cuuint64_t)T, (cuuint64_t)S};
@@ -366,6 +387,7 @@ cudaError_t launch_router_tc(const RouterArgs& a, int splits, cudaStream_t s) {
   f.E = a.E;
   f.ds = a.d / splits;
   f.N = N;
+  f.stages = lt_stages(N, f.ds / kLtKC);
   cudaError_t e = cudaSuccess;
   if (!a.parts_ready) {   // else dmoe_router_prepare wrote this W_r's parts already
     e = launch_router_wsplit(a.w_r, a.w_parts, a.d, a.E, s);
@@ -376,12 +398,12 @@ cudaError_t launch_router_tc(const RouterArgs& a, int splits, cudaStream_t s) {
   cudaGetDevice(&dev);
   if (dev >= 31 || !(mask & (1 << dev))) {
     e = cudaFuncSetAttribute(router_logits_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)lt_smem_bytes(kMaxExperts));
+                             kLtSmemMax);
     if (e != cudaSuccess) return e;
     if (dev < 31) mask |= 1 << dev;
   }
   return launch_ex(router_logits_tc_kernel, dim3((a.T + kLtM - 1) / kLtM, splits, nsplit),
-                   dim3(kLtThreads), lt_smem_bytes(N), s, true, f);
+                   dim3(kLtThreads), lt_smem_bytes(N, f.stages), s, true, f);
 }
 
 }  // namespace dmoe
