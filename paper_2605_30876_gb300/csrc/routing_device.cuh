@@ -220,7 +220,7 @@ __device__ inline void publish_coreset_mask(uint32_t* __restrict__ words, const 
 // Top-P accumulates the sorted values in order in fp32 and stops at the first running sum
 // >= p (p >= 1: at the last nonzero entry); the floor extends the coreset to k entries
 // (zero entries in id order). For p <= 0 (block top-k) the coreset is the k largest sums,
-// taken by one warp without the normalisation. For p > 0 every nonzero S~ counts the nonzero
+// taken by counting, without the normalisation. For p > 0 every nonzero S~ counts the nonzero
 // entries that beat it (larger, or equal with a lower id), all in parallel; p < 1 then adds
 // them in order up to the threshold. Needs blockDim.x == kMaxExperts.
 template <class HatFn>
@@ -283,44 +283,61 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
   if (top_p <= 0.f) {
     // p <= 0 (block top-k): Top-P stops at the first entry and the floor extends the coreset
     // to the k best. S~ = S / sum(S) has the order of S (exactly so, where the fp32 division
-    // would round two sums to one value), so the k best sums are taken directly: warp 0
-    // holds all E sums, eight per lane, and selects them by a sort and k reductions.
-    st_s[tid] = live ? S : 0.f;
-    __syncthreads();
-    if (warp == 0) {
-      float v[8];
-      int id[8];
-      uint32_t valid = 0;
+    // would round two sums to one value), so the k best sums are taken directly, by counting:
+    // a sum's place among its warp's 32 experts, then, for the k best of each warp, among those
+    // 8 k (larger key, or equal with a lower id; the id's complement is the low word).
+    // (One warp sorting eight sums a lane and popping the best k times took 0.13 us more: 16
+    // layers of one block 210.4 us against 208.3, the layer of 256 tokens 48.7 against 48.3.)
+    __shared__ __align__(16) uint64_t best[8 * kMaxTopK];
+    const uint64_t me1 = (uint64_t)(live ? order_key(S) : 0u) << 32 | (uint32_t)~tid;
+    nz_kid[tid] = me1;
+    __syncwarp();
+    int r1 = 0;
+    {
+      const ulonglong2* two = reinterpret_cast<const ulonglong2*>(nz_kid + 32 * warp);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int e = lane + 32 * j;
-        id[j] = e;
-        v[j] = e < E ? st_s[e] : 0.f;
-        if (e < E) valid |= 1u << j;
-      }
-      int my_e;
-      float my_v;
-      warp_topk(v, id, valid, k, my_e, my_v);
-      if (lane < k) order[lane] = my_e;
-      if (spec != nullptr) {
-        // block top-k: the coreset (the k best, best first) is every token's routing; it is
-        // published for the expert launch at once, three 8-bit ids and a marker byte per
-        // word, one relaxed store per word (a word reads as zero until it is complete)
-        uint32_t w = 1u << 24;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const int src = 3 * lane + j;
-          const int ej = __shfl_sync(0xffffffffu, my_e, src & 31);
-          if (src < k) w |= (uint32_t)ej << (8 * j);
-        }
-        if (lane < spec_words(k))
-          asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(spec + lane), "r"(w) : "memory");
+      for (int j = 0; j < 16; ++j) {
+        const ulonglong2 kj = two[j];
+        r1 += (kj.x > me1 ? 1 : 0) + (kj.y > me1 ? 1 : 0);
       }
     }
+    if (r1 < k) best[warp * k + r1] = me1;
     __syncthreads();
+    {
+      const int n = 8 * k, sh = k <= 8 ? 2 : 1;   // 4 or 2 threads a sum
+      const int ent = tid >> sh;
+      uint64_t me = 0;
+      int r = 0;
+      if (ent < n) {
+        me = best[ent];
+        const ulonglong2* two = reinterpret_cast<const ulonglong2*>(best);
+#pragma unroll 8
+        for (int j = tid & ((1 << sh) - 1); j < n / 2; j += 1 << sh) {
+          const ulonglong2 kj = two[j];
+          r += (kj.x > me ? 1 : 0) + (kj.y > me ? 1 : 0);
+        }
+      }
+      r += __shfl_xor_sync(0xffffffffu, r, 1);
+      if (sh == 2) r += __shfl_xor_sync(0xffffffffu, r, 2);
+      if (ent < n && (tid & ((1 << sh) - 1)) == 0 && r < k) order[r] = (int)~(uint32_t)me;
+    }
+    __syncthreads();
+    if (spec != nullptr && warp == 0) {
+      // block top-k: the coreset (the k best, best first) is every token's routing; it is
+      // published for the expert launch at once, three 8-bit ids and a marker byte per word,
+      // one relaxed store per word (a word reads as zero until it is complete)
+      uint32_t w = 1u << 24;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int src = 3 * lane + j;
+        if (src < k) w |= (uint32_t)order[src] << (8 * j);
+      }
+      if (lane < spec_words(k))
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(spec + lane), "r"(w) : "memory");
+    }
     if (coreset != nullptr && live) coreset[tid] = (tid < k) ? order[tid] : -1;
     if (coreset_size != nullptr && tid == 0) coreset_size[0] = k;
-    __syncthreads();   // st_s and order are rewritten by a later block of the same CTA
+    __syncthreads();   // the arrays and order are rewritten by a later block of the same CTA
     return k;
   }
   // Normalize: L1
@@ -335,7 +352,7 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     // id. Then one thread adds the sorted values in order until both rules are met. (Per-warp
     // sorts and a tournament over the warps' list heads, two dependent reductions per member,
     // took 3.6 us at 17 members; this 1.2. One entry a load and the key and the id compared
-    // apart: 337.4 us against 334.4 for 16 layers of one block with p = 0.6.)
+    // apart: 337.4 us against 334.8 for 16 layers of one block with p = 0.6.)
     const uint32_t key = live ? order_key(st) : 0u;
     const bool in = live && key > order_key(0.f);   // nonzero (a NaN sorts first, as its key does)
     const bool zero = live && !in;
