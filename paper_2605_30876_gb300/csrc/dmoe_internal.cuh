@@ -80,8 +80,8 @@ struct Workspace {
                        // or bf16 (general path); sized for fp32
   size_t yshared;      // [T, d], the same element type
   size_t hdense;       // bf16 [(E+1) * n_pad, max(I, I_s)]: H per group over all tokens
-  size_t spec;         // int32 [n_blocks, k]: the coreset of every block (block top-k call)
-                       // (decode-size forwards only)
+  size_t spec;         // u32 per block: its published coreset, spec_words(k) words of ids (block
+                       // top-k) or kSpecMaskWords of member bits (decode-size forwards)
   size_t disp_bits;    // u32 [ceil(T/32), E]: dispatch, token bitmap per (32-token chunk, expert)
   size_t w_parts;      // bf16 [3E, d]: split of W_r for the tcgen05 router (large forwards)
   size_t w_parts_bytes;

@@ -7,13 +7,15 @@
 // B operand of gate/up is x itself (no gather), the extra MMA columns cost nothing next to
 // the weight stream, and the down epilogue keeps only the columns of the tokens routed to
 // the group. The work is a list of units spread round-robin over one CTA per SM:
-//   gate/up unit (group, hg rows of I, hg = 64 or 32): hg rows of W_gate stacked over the
-//     same hg rows of W_up, one M = 2 hg MMA chain over K = d (gate in the first hg rows of
-//     the accumulator, up in the rest); the epilogue writes h = silu(gate) * up as bf16 into
-//     the group's H (global, L2-resident) and publishes the tile on the group's counter;
+//   gate/up unit (group, hg rows of I, hg = 64 or 32): hg rows of W_gate and the same hg rows
+//     of W_up, eight of each in turn (one box of a map over both tensors, or a box per eight
+//     rows where their distance has no map), one M = 2 hg MMA chain over K = d; gate and up of
+//     a row lie eight lanes apart in one warp, which exchange them by shuffles and write
+//     h = silu(gate) * up as bf16 into the group's H (global, L2-resident); the tile is then
+//     published on the group's counter;
 //   down unit (group, 128 rows of d): D = W_down tile x H^T over K = I; the producer loads
 //     the weight stages first and the H stages once every gate/up tile of the group is
-//     published; the epilogue stores the fp32 rows per (token, slot).
+//     published; the epilogue stores the fp32 rows per (token, slot), eight columns at a time.
 // Down units continue the round-robin where the gate/up units stopped. hg is chosen on the
 // device once the unique-expert count is known: 32 when the 32-row gate/up units still fit
 // in one round over the CTAs, else 64. With few unique experts the 64-row units would
@@ -55,11 +57,12 @@ constexpr int kMaxTok = 64;                     // tokens of a decode-sized forw
 // g_dtrace[cta * 32 + slot] (globaltimer ns): 0 entry, 1 unit list known, 2 gate/up first
 // stage landed, 3 gate/up MMAs committed, 4 gate/up tile published, 5 down weights issued,
 // 6 H ready seen, 7 down MMAs committed, 8 down rows stored, 9 exit, 10 gate/up unit id,
-// 11 down unit id, 12/13 first/last down stage landed, 14 down accumulator ready, 15 down
-// accumulator staged, 16 staging complete, 17 row copies issued, 18 coresets seen by the
-// polling warp, 19 its CTA past the barrier after the poll, 26/27 fourth / last gate/up
-// stage landed, 28/29 first / last gate/up stage issued, 30 past the TMEM barrier, 31 the
-// producer's cache policies made.
+// 11 down unit id, 12/13 first/last down stage landed, 14 down accumulator ready, 15 its rows
+// stored by the first warp, 18 coresets seen by the polling warp, 19 its CTA past the barrier
+// after the poll, 20 gate/up accumulator ready, 21 / 22 H box staged / stored, 23 accumulator
+// read, 25 SwiGLU done, 26/27 fourth / last gate/up stage landed, 28/29
+// first / last gate/up stage issued, 30 past the TMEM barrier, 31 the producer's cache policies
+// made.
 #ifdef DMOE_TRACE
 __device__ uint64_t g_dtrace[kMaxPersistentCtas * 32];
 #define ED_AT(slot) (g_dtrace[blockIdx.x * 32 + (slot)] = ptx::globaltimer_ns())

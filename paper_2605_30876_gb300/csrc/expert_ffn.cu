@@ -60,13 +60,11 @@ constexpr int kRowStages = 5;                      // ring slots of the token ro
 constexpr int kProgress = 64;                      // steps (K = 128) whose completion is remembered
 constexpr int kQueue = 4;                          // units handed out and not yet taken up by every role
 constexpr int kSpecBlocks = 64;                    // blocks of a block top-k forward, at most
-constexpr int kSpecPairs = kSpecBlocks * kMaxTopK;   // (block, coreset member) pairs, at most
 
 struct GemmParams {
   const int32_t* n_unique;
   const int32_t* unique_ids;
   const int32_t* offsets;
-  const int32_t* rows;    // dispatch rows: t * k + slot (the x row of a routed token row)
   __nv_bfloat16* h;       // [T*k, I]
   __nv_bfloat16* hs;      // [T, Is]
   __nv_bfloat16* yslot;   // [T*k, d] bf16 (the combine sums them in fp32)
@@ -76,7 +74,7 @@ struct GemmParams {
   DevErrRecord* err;
   const void* ws_gate; const void* ws_up; const void* ws_down;  // shared, prefetched if set
   int T, d, E, k, I, Is;
-  int n_max;              // token tile, at most; a multiple of
+  int n_max;              // token tile, at most; a multiple of `unit`
   int unit;               // rows that every tile is a multiple of (expert_tile_unit(blk) or 32)
   int box[kLevels];       // rows of the token row boxes: n_max / 2 (a CTA's half), and smaller
   int ntiles;             // token tiles per group at most
@@ -209,12 +207,10 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   int* g_row0 = dn_prefix + (kMaxGroups + 1);      // by group
   int* g_cnt = g_row0 + kMaxGroups;
   int* g_e = g_cnt + kMaxGroups;
-  // block top-k planning: blocks per expert (bit b of s_bmask[2e + b / 32]), each block's
-  // coreset, per expert its group and the blocks of the groups before it
+  // block top-k planning: blocks per expert (bit b of s_bmask[2e + b / 32]) and the blocks of
+  // the groups before its own
   uint32_t* s_bmask = reinterpret_cast<uint32_t*>(g_e + kMaxGroups);   // [2 * kMaxExperts]
-  int16_t* s_upos = reinterpret_cast<int16_t*>(s_bmask + 2 * kMaxExperts);   // [kMaxExperts]
-  int16_t* s_bpos = s_upos + kMaxExperts;                                      // [kMaxExperts]
-  uint8_t* s_bcore = reinterpret_cast<uint8_t*>(s_bpos + kMaxExperts);   // [kSpecPairs]
+  int16_t* s_bpos = reinterpret_cast<int16_t*>(s_bmask + 2 * kMaxExperts);   // [kMaxExperts]
 
   constexpr bool spec = kSpec;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -298,7 +294,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
             if (e >= p.E) {
               bad = true;
             } else {
-              s_bcore[b * p.k + r0 + j] = (uint8_t)e;
               atomicOr(&s_bmask[2 * e + (b >> 5)], 1u << (b & 31));
             }
           }
@@ -334,7 +329,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       for (int q = 0; q < 8; ++q)
         if (nbq[q] > 0) {
           const int e = 8 * lane + q;
-          s_upos[e] = (int16_t)u;
           s_bpos[e] = (int16_t)bp;
           g_e[u] = e;
           g_row0[u] = p.blk * bp;
@@ -1161,7 +1155,7 @@ uint32_t pow2_cols(uint32_t c) {
 size_t experts_fixed_smem() {
   // alignment slack + barriers + misc/group arrays + block top-k planning
   return 1024 + 8 * (kMaxStages + kRowStages + kProgress + 9 + 5 * kQueue) + sizeof(int) * (12 + 5 * (kMaxGroups + 1)) +
-         64 + 4 * 2 * kMaxExperts + 2 * 2 * kMaxExperts + kSpecPairs;
+         64 + 4 * 2 * kMaxExperts + 2 * kMaxExperts;
 }
 
 int max_smem_optin() {

@@ -469,13 +469,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void*
       "r"(smem_addr(src)), "r"(x), "r"(y), "r"(z)
       : "memory");
 }
-// 1-D bulk copy of `bytes` (multiple of 16, both addresses 16-B aligned) from shared to
-// global memory, tracked by a bulk group
-__device__ __forceinline__ void bulk_store(void* gdst, const void* ssrc, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst),
-               "r"(smem_addr(ssrc)), "r"(bytes)
-               : "memory");
-}
 // commits the bulk copies issued so far and waits until they are complete
 __device__ __forceinline__ void bulk_commit_wait_all() {
   asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group 0;" ::: "memory");
