@@ -95,7 +95,8 @@ struct DParams {
   int h32_ok;                // 32-row gate/up units allowed (d % 256 == 0, >= 3 slots fit)
   int has_shared;
   int gu_box, sgu_box;       // gate and up rows come in one box (DMaps::gu ..): 1: gate first, 2:
-                             // up first; 0: a box per 8 rows (routed experts, shared expert)
+                             // up first (routed experts, shared expert)
+  int far;                   // ... or in boxes of their own, gate first (DMaps::wg ..), in both
   int n_acc;                 // TMEM accumulators of n_pad columns
   uint32_t tmem_cols;
 };
@@ -103,9 +104,10 @@ struct DParams {
 // Every map sees its matrix as [K / 64][rows][64], so that one copy brings a whole stage (several
 // 64-column K boxes): the producer issues two copies per stage, weights and token rows.
 struct DMaps {
-  CUtensorMap gu, sgu;       // gate/up, [K / 64][rows / 8][2][8][64]: 64 rows of each (K = 128)
+  CUtensorMap gu, sgu;       // gate/up, [rows / 8][2][K / 64][8][64]: 64 rows of each (K = 128)
   CUtensorMap gu32, sgu32;   // ... 32 rows of each (K = 256)
-  CUtensorMap wg, wu, sg, su;   // ... 8 rows of one (K = 64)
+  CUtensorMap wg, wu, sg, su;           // one tensor, [rows / 8][K / 64][8][64]: 16 rows, K = 128
+  CUtensorMap wg32, wu32, sg32, su32;   // ... 8 rows, K = 256
   CUtensorMap wd, sd;        // down: 128 rows, K = 128
   CUtensorMap x, x32;        // x [T, d]: n_pad rows (rows >= T read as zeros), K = 128 / 256
   CUtensorMap h;             // hdense: n_pad rows, K = 128 (down B operand)
@@ -133,22 +135,25 @@ using ptx::tma_store_2d;
 __device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __expf(-z)); }
 
 // One gate/up stage's weights: hg (32 or 64) rows of W_gate and the same rows of W_up from row
-// arow, 8 of each in turn, over the 64-column K boxes from kb on (32 KB).
+// arow, some of each in turn (gate_rows), over the 64-column K boxes from kb on (32 KB): each 8
+// rows over all K boxes of the stage, 1 KB a box. Tensors too far apart for one map (allocations
+// in two address ranges) take 8 copies of 4 KB (98 unique experts, I = 384: one map 87 us, 32
+// copies of 1 KB 150, 16 of 2 KB 113).
 __device__ __forceinline__ void load_gate_up(const DMaps& tm, const DParams& p, uint8_t* dst,
                                              uint64_t* bar, bool shared, bool h32, int arow, int kb,
                                              uint64_t pol) {
-  if ((shared ? p.sgu_box : p.gu_box) != 0) {
+  if (!p.far) {
     const CUtensorMap* m = shared ? (h32 ? &tm.sgu32 : &tm.sgu) : (h32 ? &tm.gu32 : &tm.gu);
-    ptx::tma_load_5d(dst, m, bar, 0, 0, 0, arow / kGateRows, kb, pol);
+    ptx::tma_load_5d(dst, m, bar, 0, 0, kb, 0, arow / kGateRows, pol);
     return;
   }
-  const int hg = h32 ? 32 : 64;
-  for (int b = 0; b < kTileM / hg; ++b)
-    for (int r = 0; r < hg; r += kGateRows, dst += 2 * kGateRows * 128) {
-      ptx::tma_load_3d(dst, shared ? &tm.sg : &tm.wg, bar, 0, arow + r, kb + b, pol);
-      ptx::tma_load_3d(dst + kGateRows * 128, shared ? &tm.su : &tm.wu, bar, 0, arow + r, kb + b,
-                       pol);
-    }
+  const CUtensorMap* mg = shared ? (h32 ? &tm.sg32 : &tm.sg) : (h32 ? &tm.wg32 : &tm.wg);
+  const CUtensorMap* mu = shared ? (h32 ? &tm.su32 : &tm.su) : (h32 ? &tm.wu32 : &tm.wu);
+  for (int j = 0; j < 4; ++j, dst += kAStage / 4) {
+    const int r8 = arow / 8 + (h32 ? j : 2 * j);
+    ptx::tma_load_4d(dst, mg, bar, 0, 0, kb, r8, pol);
+    ptx::tma_load_4d(dst + kAStage / 8, mu, bar, 0, 0, kb, r8, pol);
+  }
 }
 
 // kMask: the coresets are published as masks (DParams::spec_mask), compiled separately so
@@ -350,7 +355,6 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
   const int S = h32 ? S32 : S64;
   auto slot_a = [&](int st) { return ring + st * slot; };
   auto slot_b = [&](int st) { return ring + st * slot + kAStage; };
-  const int abox_g = 2 * hg * 128;                // one K box of the stacked gate|up rows
   const int ngu_s = h32 ? ngu_s32 : ngu64_s, ngu_r = h32 ? ngu_r32 : ngu64_r;
   const int NGU = ngu_s + U * ngu_r;
   const int ND = G * ndn;
@@ -551,8 +555,10 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     int stage = 0, acc = 0;
     uint32_t phase = 0, acc_phase = 0;
     bool ok = true, first = half == 0;
-    // nstages stages of kboxes K boxes each; A boxes abox bytes apart, M = mrows
-    auto run = [&](int nstages, int kboxes, int abox, uint32_t mrows, int value, bool gu) {
+    // nstages stages of kboxes K boxes each; A's K boxes abox bytes apart, its groups of eight
+    // rows sbo, M = mrows
+    auto run = [&](int nstages, int kboxes, int abox, uint32_t sbo, uint32_t mrows, int value,
+                   bool gu) {
       const uint32_t n_mma = (uint32_t)((p.T + 15) & ~15);
       const uint32_t idesc = ptx::idesc_bf16(mrows, n_mma);
       if (!wait(&acc_empty[acc], acc_phase ^ 1u, value)) { ok = false; return; }
@@ -572,7 +578,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
         for (int kb = kb0; kb < kb1; ++kb)
 #pragma unroll
           for (int kk = 0; kk < kTileK / 16; ++kk)
-            ptx::mma_bf16(d0, ptx::sdesc_k_sw128(a0 + kb * abox + kk * 32),
+            ptx::mma_bf16(d0, ptx::sdesc_k_sw128(a0 + kb * abox + kk * 32, sbo),
                           ptx::sdesc_k_sw128(b0 + kb * bbox + kk * 32), idesc,
                           (c > 0 || kb > kb0 || kk > 0) ? 1u : 0u);
         ptx::mma_commit(&empty[stage]);
@@ -585,14 +591,14 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       int gi, m;
       gu_unit(u, gi, m);
       // all T token columns: the B box is x (rows >= T are zeros)
-      run(kc, kbg, abox_g, (uint32_t)(2 * hg), u, true);
+      run(kc, kbg, kGateRows * 128, (uint32_t)(kbg * kGateRows * 128), (uint32_t)(2 * hg), u, true);
       if (first) ED_AT(3);
       first = false;
     }
     first = half == 0;
     for (int v = v0; v < ND && ok; v += nb) {
       const Grp g = group_w(v / ndn);
-      run(g.Ig / kStageK, kKB, kABox, (uint32_t)kTileM, v, false);
+      run(g.Ig / kStageK, kKB, kABox, 1024u, (uint32_t)kTileM, v, false);
       if (first) ED_AT(7);
       first = false;
     }
@@ -609,9 +615,13 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     // gate/up accumulator (M = 2 hg): row r sits in TMEM lane r for M = 128 and in lane
     // 32 (r / 16) + r % 16 for M = 64. The A tile holds 8 gate rows and the same 8 up rows in
-    // turn, so the up row of a gate lane l is in lane l + 8 of the same warp
+    // turn (16 for M = 128 from tensors far apart), so the up row of a gate lane l is in lane
+    // l + 8 (16) of the same warp
     const bool g_act = hg == 64 || lane < 16;
-    const int rr = (hg == 64 ? 16 * q + 8 * (lane >> 4) : 8 * q) + (lane & 7);   // row of the tile
+    const int gate_rows = p.far && hg == 64 ? 16 : kGateRows;
+    // row of the tile
+    const int rr = hg != 64 ? 8 * q + (lane & 7)
+                            : 16 * q + (p.far ? lane & 15 : 8 * (lane >> 4) + (lane & 7));
     const int n_mma = (p.T + 15) & ~15;
     const uint32_t part1 = (uint32_t)(p.n_acc * p.n_pad);   // column offset of part 1
     // 16 columns of an accumulator: the sum of its two parts
@@ -642,7 +652,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       // gives its last 8 columns to the lane that holds its row's up values and takes that
       // one's first 8; each then has gate and up of one row for 8 tokens
       const bool gate_first = (gi < p.has_shared ? p.sgu_box : p.gu_box) != 2;
-      const bool is_gate = ((lane & 8) == 0) == gate_first;
+      const bool is_gate = ((lane & gate_rows) == 0) == gate_first;
       uint8_t* hdst = hbox + (rr >> 5) * p.n_pad * 64 + (rr & 30) * 2;
       for (int c0 = 0; c0 < n_mma; c0 += 16) {
         float v[16];
@@ -652,7 +662,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const float other =
-              __shfl_xor_sync(0xffffffffu, is_gate ? v[8 + j] : v[j], kGateRows);
+              __shfl_xor_sync(0xffffffffu, is_gate ? v[8 + j] : v[j], gate_rows);
           h[j] = silu_f(is_gate ? v[j] : other) * (is_gate ? other : v[8 + j]);
         }
         uint32_t w[4];
@@ -812,15 +822,29 @@ int make_map_two(CUtensorMap* m, const void* a, const void* b, uint64_t rows, ui
   const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
   const uint64_t dist = pa < pb ? pb - pa : pa - pb;
   if (enc == nullptr || dist == 0 || dist % 16 != 0 || dist >= ((uint64_t)1 << 40)) return 0;
-  const cuuint64_t dims[5] = {64, kGateRows, 2, rows / kGateRows, cols / 64};
-  const cuuint64_t strides[4] = {cols * 2, dist, cols * 2 * kGateRows, 128};
-  const cuuint32_t box[5] = {64, kGateRows, 2, hg / kGateRows, ksteps};
+  const cuuint64_t dims[5] = {64, kGateRows, cols / 64, 2, rows / kGateRows};
+  const cuuint64_t strides[4] = {cols * 2, 128, dist, cols * 2 * kGateRows};
+  const cuuint32_t box[5] = {64, kGateRows, ksteps, 2, hg / kGateRows};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   if (enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pa < pb ? a : b), dims, strides,
           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return 0;
   return pa < pb ? 1 : 2;
+}
+
+// One matrix as [rows / 8][cols / 64][8][64]: a box of box_rows rows, each 8 over `ksteps` steps.
+bool make_map_far(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols,
+                  uint32_t box_rows, uint32_t ksteps) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  const cuuint64_t dims[4] = {64, 8, cols / 64, rows / 8};
+  const cuuint64_t strides[3] = {cols * 2, 128, cols * 16};
+  const cuuint32_t box[4] = {64, 8, ksteps, box_rows / 8};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // bf16 matrix [rows, cols] row-major, box = 32 columns x box_rows rows, no swizzle.
@@ -919,17 +943,24 @@ cudaError_t launch_experts_decode(const ExpertArgs& a, cudaStream_t s) {
     if (p.gu_box != 0)
       p.gu_box = make_map_two(&m.gu32, a.w_gate, a.w_up, gu_rows, a.d, 32, kTileM / 32);
   }
-  if (p.gu_box == 0)
-    ok = ok && make_map(&m.wg, a.w_gate, gu_rows, a.d, kGateRows, 1) &&
-         make_map(&m.wu, a.w_up, gu_rows, a.d, kGateRows, 1);
   if (has_shared) {
     ok = ok && make_map(&m.sd, a.ws_down, (uint64_t)a.d, a.Is, kTileM, kKB);
     p.sgu_box = make_map_two(&m.sgu, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d, 64, kTileM / 64);
     if (ring.h32_ok && p.sgu_box != 0)
       p.sgu_box = make_map_two(&m.sgu32, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d, 32, kTileM / 32);
-    if (p.sgu_box == 0)
-      ok = ok && make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, kGateRows, 1) &&
-           make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, kGateRows, 1);
+  }
+  // tensors too far apart for one map: all of them in boxes of their own
+  p.far = p.gu_box == 0 || (has_shared && p.sgu_box == 0) ? 1 : 0;
+  if (p.far) {
+    p.gu_box = p.sgu_box = 0;
+    auto apart = [&](CUtensorMap* m64, CUtensorMap* m32, const void* w, uint64_t rows) {
+      return make_map_far(m64, w, rows, a.d, 16, 2) &&
+             (!ring.h32_ok || make_map_far(m32, w, rows, a.d, 8, 4));
+    };
+    ok = ok && apart(&m.wg, &m.wg32, a.w_gate, gu_rows) && apart(&m.wu, &m.wu32, a.w_up, gu_rows);
+    if (has_shared)
+      ok = ok && apart(&m.sg, &m.sg32, a.ws_gate, (uint64_t)a.Is) &&
+           apart(&m.su, &m.su32, a.ws_up, (uint64_t)a.Is);
   }
   if (!ok) return cudaErrorInvalidValue;
 

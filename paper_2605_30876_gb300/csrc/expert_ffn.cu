@@ -85,7 +85,7 @@ struct GemmParams {
   uint32_t tmem_cols;
   int has_shared;
   int gu_box, sgu_box;    // gate and up rows come in one box (Maps::gu / sgu): 1: gate first,
-                          // 2: up first; 0: a box per 16 rows (routed experts, shared expert)
+                          // 2: up first; 0 (both): a box per 16 rows (routed, shared expert)
   // Block top-k (spec_words != nullptr): the groups come from the coresets that the block
   // routing launch publishes (n_blocks blocks of blk rows). The unique experts are their
   // union, ascending; an expert's token rows are its blocks' rows in block order, which is
@@ -104,7 +104,8 @@ struct GemmParams {
 // Weights and the shared expert's rows: [rows, K] in boxes of 64 columns (K). Routed token rows:
 // [rows, K] seen as [K / 64][rows][64], so that one box brings several K steps of few rows.
 struct Maps {
-  CUtensorMap wg, wu, sg, su;   // gate/up weights, 16-row boxes (routed [E*I,d], shared [Is,d])
+  CUtensorMap wg, wu, sg, su;   // gate/up weights apart: [rows / 8][K / 64][8][64], 16 rows and
+                                // K = 128 in one box (routed [E*I,d], shared [Is,d])
   CUtensorMap gu, sgu;          // both at once: [rows / 16][2][16][d], 64 rows of each in one box
   CUtensorMap wd, sd;           // down weights, 128-row boxes (routed [E*d,I], shared [d,Is])
   CUtensorMap x, hs;            // shared expert's token rows: x [T,d], Hs [T,Is]
@@ -171,8 +172,11 @@ __device__ uint64_t g_trace[kMaxPersistentCtas * 64];
 // loaded as ring slots free; only its token rows wait (bounded) for the gate/up tiles of those
 // rows to be published (h_ready), so weight streaming of both phases overlaps. kSpec: the block
 // top-k form (GemmParams::spec_words), compiled separately so that the other form carries none
-// of its code.
-template <bool kSpec>
+// of its code. kFar: W_gate and W_up too far apart for one map (2^40 bytes or more: allocations
+// in two address ranges; or the same tensor), 16 rows of each over K = 128 in a box of their own,
+// filling two slots. 256 tokens, token routing, 128 experts of I = 384: 110 us with one map, 125
+// so, 137 with 16 rows over K = 64 a box (2 KB copies are below the HBM rate).
+template <bool kSpec, bool kFar>
 __global__ void __launch_bounds__(kThreads, 1)
 moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -239,7 +243,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     *s_rows_ok = 0;
     ptx::fence_mbarrier_init();
     *s_abort = 0;
-    ptx::prefetch_tensormap(&tm.gu);
+    ptx::prefetch_tensormap(kFar ? &tm.wg : &tm.gu);
     ptx::prefetch_tensormap(&tm.wd);
     ptx::prefetch_tensormap(spec ? &tm.xb : &tm.xp[0]);
     ptx::prefetch_tensormap(&tm.h[0]);
@@ -569,7 +573,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         // stores nothing)
         const int arow = un.gu ? (shared ? 0 : g_e[un.g] * p.I) + un.m * 128 + rank * 64
                                : (shared ? 0 : g_e[un.g] * p.d) + un.m * 256 + rank * kTileM;
-        const int one_box = shared ? p.sgu_box : p.gu_box;
         const CUtensorMap* m0 = un.gu ? (shared ? &tm.sg : &tm.wg) : (shared ? &tm.sd : &tm.wd);
         const CUtensorMap* m1 = shared ? &tm.su : &tm.wu;
         const CUtensorMap* m01 = shared ? &tm.sgu : &tm.gu;
@@ -581,13 +584,14 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
           const uint32_t bar = full0 + 8u * (uint32_t)stage;
           if (!un.gu) {
             ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow, pol_w);
-          } else if (one_box != 0) {
+          } else if (!kFar) {
             ptx::tma_load_4d_pair(dst, m01, bar, c * kTileK, 0, 0, arow / kGateRows, pol_w);
-          } else {
-            for (int r = 0; r < 64; r += kGateRows, dst += 2 * kGateRows * 128) {
-              ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow + r, pol_w);
-              ptx::tma_load_2d_pair(dst + kGateRows * 128, m1, bar, c * kTileK, arow + r, pol_w);
-            }
+          } else if ((c & 1) == 0) {   // two slots at once (their number is even)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              ptx::tma_load_4d_pair(dst + j * 2 * kGateRows * 128, (j & 1) ? m1 : m0,
+                                    bar + 8u * (uint32_t)(j / 4), 0, 0, c,
+                                    arow / 8 + (j >> 1) * (kGateRows / 8), pol_w);
           }
           if (++stage == a_stages) { stage = 0; phase ^= 1u; }
           if (rank == 0 && c == kc / 2) {
@@ -758,7 +762,13 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
 #pragma unroll
             for (int k2 = 0; k2 < 2; ++k2) {
               ok = ok && (a_in || wait(&a_full[sa], pa, i));
-              const uint32_t as = a0 + (uint32_t)sa * kATileBytes;
+              uint32_t as = a0 + (uint32_t)sa * kATileBytes;
+              uint32_t sbo = 1024u;
+              if (kFar && un.gu) {    // two slots hold the step: rows of 8 over both K boxes
+                if (k2 == 0) ok = ok && wait(&a_full[sa + 1], pa, i);
+                as = a0 + (uint32_t)(sa - k2) * kATileBytes + (uint32_t)k2 * 1024u;
+                sbo = 2048u;
+              }
               if (++sa == a_stages) { sa = 0; pa ^= 1u; }
               bs += step_bytes;
               if (++kb == kpb) {      // the next slot
@@ -771,7 +781,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
               ptx::tc_fence_after();
 #pragma unroll
               for (int kk = 0; kk < kTileK / 16; ++kk) {
-                ptx::mma_bf16_pair(d0, ptx::sdesc_k_sw128(as + kk * 32),
+                ptx::mma_bf16_pair(d0, ptx::sdesc_k_sw128(as + kk * 32, sbo),
                                    ptx::sdesc_k_sw128(bs + kk * 32), idesc,
                                    (c > 0 || k2 > 0 || kk > 0) ? 1u : 0u);
                 if (kk == 1) {
@@ -1146,6 +1156,20 @@ int make_map_two(CUtensorMap* m, const void* a, const void* b, uint64_t rows, ui
   return pa < pb ? 1 : 2;
 }
 
+// One matrix as [rows / 8][cols / 64][8][64]: a box of 16 rows and K = 128, each 8 rows over both
+// K boxes (4 KB a copy, where 2 KB over one K box leave the copy engine short of the HBM rate).
+bool make_map_far(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols) {
+  EncodeTiledFn enc = encode_fn();
+  if (enc == nullptr) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)kTileK, 8, cols / kTileK, rows / 8};
+  const cuuint64_t strides[3] = {cols * 2, (cuuint64_t)kTileK * 2, cols * 16};
+  const cuuint32_t box[4] = {(cuuint32_t)kTileK, 8, 2, kGateRows / 8};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 uint32_t pow2_cols(uint32_t c) {
   uint32_t r = 32;
   while (r < c) r <<= 1;
@@ -1250,9 +1274,6 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   const uint64_t gu_rows = (uint64_t)a.E * a.I;
   bool ok = make_map(&m.wd, a.w_down, (uint64_t)a.E * a.d, a.I, kTileM);
   gp.gu_box = make_map_two(&m.gu, a.w_gate, a.w_up, gu_rows, a.d);
-  if (gp.gu_box == 0)
-    ok = ok && make_map(&m.wg, a.w_gate, gu_rows, a.d, kGateRows) &&
-         make_map(&m.wu, a.w_up, gu_rows, a.d, kGateRows);
   if (spec) ok = ok && make_map(&m.xb, a.x, (uint64_t)a.T, a.d, (uint32_t)gp.blk);
   for (int i = 0; i < kLevels; ++i) {
     const uint32_t rows = (uint32_t)gp.box[i], ksteps = (uint32_t)(gp.box[0] / gp.box[i]);
@@ -1264,9 +1285,16 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
          make_map(&m.x, a.x, (uint64_t)a.T, a.d, (uint32_t)gp.box[0]) &&
          make_map(&m.hs, a.hs, (uint64_t)a.T, a.Is, (uint32_t)gp.box[0]);
     gp.sgu_box = make_map_two(&m.sgu, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d);
-    if (gp.sgu_box == 0)
-      ok = ok && make_map(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d, kGateRows) &&
-           make_map(&m.su, a.ws_up, (uint64_t)a.Is, a.d, kGateRows);
+  }
+  // tensors too far apart for one map (the form with a box per 16 rows then loads all of them)
+  const bool far = gp.gu_box == 0 || (has_shared && gp.sgu_box == 0);
+  if (far) {
+    gp.gu_box = gp.sgu_box = 0;
+    ok = ok && make_map_far(&m.wg, a.w_gate, gu_rows, a.d) &&
+         make_map_far(&m.wu, a.w_up, gu_rows, a.d);
+    if (has_shared)
+      ok = ok && make_map_far(&m.sg, a.ws_gate, (uint64_t)a.Is, a.d) &&
+           make_map_far(&m.su, a.ws_up, (uint64_t)a.Is, a.d);
   }
   if (!ok) return cudaErrorInvalidValue;
 
@@ -1283,6 +1311,7 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   // start while it runs)
   const int most = spec ? kMaxStages - 4 : kMaxStages;
   if (gp.a_stages > most) gp.a_stages = most;
+  if (far) gp.a_stages &= ~1;
   if (gp.a_stages < 2) return cudaErrorInvalidConfiguration;
   gp.acc_cols = pow2_cols((uint32_t)a.n_max);
   gp.n_acc = 512 / (int)gp.acc_cols;
@@ -1293,11 +1322,11 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 31 || !(attr_dev_mask & (1 << dev))) {
-    cudaError_t e = cudaFuncSetAttribute(moe_experts_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(moe_experts_kernel<true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
+    cudaError_t e = cudaSuccess;
+    for (auto* kernel : {moe_experts_kernel<false, false>, moe_experts_kernel<true, false>,
+                         moe_experts_kernel<false, true>, moe_experts_kernel<true, true>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
     if (dev < 31) attr_dev_mask |= 1 << dev;
   }
@@ -1305,7 +1334,9 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   if (grid > kMaxPersistentCtas) grid = kMaxPersistentCtas;
   if (grid < kCluster) return cudaErrorInvalidConfiguration;
   prof_begin(DMOE_KERNEL_EXPERTS, s);
-  cudaError_t e = launch_cluster(spec ? moe_experts_kernel<true> : moe_experts_kernel<false>,
+  cudaError_t e = launch_cluster(far ? (spec ? moe_experts_kernel<true, true> : moe_experts_kernel<false, true>)
+                                     : (spec ? moe_experts_kernel<true, false>
+                                             : moe_experts_kernel<false, false>),
                                  dim3(grid), dim3(kThreads), smem, s, kCluster,
                                  !prof_serial(DMOE_KERNEL_EXPERTS), m, gp);
   prof_end(DMOE_KERNEL_EXPERTS, s);

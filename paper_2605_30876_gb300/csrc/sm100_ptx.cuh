@@ -114,6 +114,16 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(x), "r"(y), "r"(z), "l"(policy)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                            int32_t x, int32_t y, int32_t z, int32_t w,
+                                            uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_addr(bar)), "r"(x), "r"(y), "r"(z), "r"(w),
+      "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, uint64_t* bar,
                                             int32_t x, int32_t y, int32_t z, int32_t w, int32_t v,
                                             uint64_t policy) {
@@ -376,13 +386,13 @@ __device__ __forceinline__ void tmem_ld_wait() {
 }
 
 // Shared-memory matrix descriptor: K-major operand stored as rows of 128 B (64 bf16) with
-// the 128-byte swizzle, 8-row core groups 1024 B apart (SBO); the tile base must be
+// the 128-byte swizzle, 8-row core groups `sbo` bytes apart (SBO); the tile base must be
 // 1024-B aligned. Advancing K by 16 elements inside the 128-B row adds 32 B to the start.
-__device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr) {
+__device__ __forceinline__ uint64_t sdesc_k_sw128(uint32_t saddr, uint32_t sbo = 1024u) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);  // start address
   d |= (uint64_t)1 << 16;                    // leading byte offset (unused for this layout)
-  d |= (uint64_t)(1024u >> 4) << 32;         // stride byte offset
+  d |= (uint64_t)(sbo >> 4) << 32;           // stride byte offset
   d |= (uint64_t)1 << 46;                    // descriptor version for tcgen05
   d |= (uint64_t)2 << 61;                    // 128-byte swizzle
   return d;
