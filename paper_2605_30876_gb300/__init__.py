@@ -111,6 +111,10 @@ def _load() -> ctypes.CDLL:
 
 _lib = _load()
 
+_Tensor = torch.Tensor
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = torch._C._cuda_getDevice if _raw_stream is not None else None
+
 
 def _check(status: int, where: str) -> None:
     if status != DMOE_OK:
@@ -120,24 +124,25 @@ def _check(status: int, where: str) -> None:
 
 def _ptr(t, dtype=None, name="tensor"):
     """Device pointer of a contiguous CUDA tensor (None -> NULL; an int is passed through)."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    if not isinstance(t, torch.Tensor):
+    if not isinstance(t, _Tensor):
+        if t is None or isinstance(t, int):
+            return t
         raise TypeError(f"{name}: expected a torch.Tensor")
     if not t.is_cuda:
         raise ValueError(f"{name}: must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name}: must be contiguous")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise TypeError(f"{name}: expected {dtype}, got {t.dtype}")
     return t.data_ptr()
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None or not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        # the same stream without the Python object that torch.cuda.current_stream() makes
+        return _raw_stream(_current_device())
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
