@@ -133,8 +133,8 @@ Workspace plan_workspace(const dmoe_layer_desc& d) {
   w.hdense = take(dec ? 2 * (E + 1) * (size_t)((T + 15) / 16 * 16) * (I > Is ? I : Is) : 0);
   w.spec = take(dec || d.mode == DMOE_ROUTE_BLOCK
                     ? sizeof(uint32_t) * d.n_blocks *
-                          (spec_words((int)k) > kSpecMaskWords ? spec_words((int)k)
-                                                               : kSpecMaskWords)
+                          (dec && kSpecMaskWords > spec_words((int)k) ? kSpecMaskWords
+                                                                      : spec_words((int)k))
                     : 0);
   const size_t nchunks = (T + 31) / 32;
   w.disp_bits = take(sizeof(uint32_t) * nchunks * E);

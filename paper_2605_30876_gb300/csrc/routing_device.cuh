@@ -286,7 +286,7 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     // would round two sums to one value), so the k best sums are taken directly, by counting:
     // a sum's place among its warp's 32 experts, then, for the k best of each warp, among those
     // 8 k (larger key, or equal with a lower id; the id's complement is the low word).
-    // (One warp sorting eight sums a lane and popping the best k times took 0.13 us more: 16
+    // (One warp sorting eight sums a lane and popping the best k times took 0.26 us more: 8
     // layers of one block 210.4 us against 208.3, the layer of 256 tokens 48.7 against 48.3.)
     __shared__ __align__(16) uint64_t best[8 * kMaxTopK];
     const uint64_t me1 = (uint64_t)(live ? order_key(S) : 0u) << 32 | (uint32_t)~tid;
@@ -352,7 +352,7 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     // id. Then one thread adds the sorted values in order until both rules are met. (Per-warp
     // sorts and a tournament over the warps' list heads, two dependent reductions per member,
     // took 3.6 us at 17 members; this 1.2. One entry a load and the key and the id compared
-    // apart: 337.4 us against 334.8 for 16 layers of one block with p = 0.6.)
+    // apart: 337.4 us against 334.8 for 8 layers of one block with p = 0.6.)
     const uint32_t key = live ? order_key(st) : 0u;
     const bool in = live && key > order_key(0.f);   // nonzero (a NaN sorts first, as its key does)
     const bool zero = live && !in;
