@@ -145,13 +145,16 @@ dispatch_place_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
       }
     }
   }
-  int total_pairs = 0;
-  const int off = block_exclusive_scan_i(cnt, iscr, &total_pairs);
+  // rows before each expert's (at most 65536: 20 bits) and the experts with rows before it, in
+  // one scan
+  static_assert(kMaxTokens * kMaxTopK < (1 << 20) && kMaxExperts < (1 << 11), "packed scan");
+  int total = 0;
+  const int present = cnt > 0 ? 1 : 0;
+  const int scan = block_exclusive_scan_i(cnt | present << 20, iscr, &total);
+  const int off = scan & 0xfffff;
   base[tid] = off + before;
   if (first) {
-    int n_u = 0;
-    const int present = cnt > 0 ? 1 : 0;
-    const int upos = block_exclusive_scan_i(present, iscr, &n_u);
+    const int upos = scan >> 20, n_u = total >> 20, total_pairs = total & 0xfffff;
     if (present) {
       unique_ids[upos] = tid;
       offsets[upos] = off;
