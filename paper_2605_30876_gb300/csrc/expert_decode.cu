@@ -48,7 +48,9 @@ constexpr int kStageK = kKB * kTileK;
 constexpr int kABox = kTileM * 128;             // 128 rows x 128 B (W_down)
 constexpr int kAStage = kKB * kABox;            // 32 KB of weights in every stage
 constexpr int kMaxKBG = 4;                      // K boxes per gate/up stage (hg = 32)
-constexpr int kMaxStagesD = 6;
+// ring slots at most (up to 16 tokens six would fit; four layers with token routing, six / five:
+// 16 tokens 448 / 440 us and 334 / 330, 8 tokens 287 / 288 and 241 / 239)
+constexpr int kMaxStagesD = 5;
 constexpr int kGateRows = 8;                    // rows of W_gate, then of W_up, in an A tile
 constexpr uint64_t kTimeoutNs = 1000000000ull;  // 1 s
 constexpr int kMaxTok = 64;                     // tokens of a decode-sized forward
