@@ -39,6 +39,7 @@
 #include <mutex>
 
 #include "dmoe_internal.cuh"
+#include "silu.cuh"
 #include "sm100_ptx.cuh"
 #include "trace_log.cuh"
 
@@ -119,9 +120,6 @@ using ptx::ld_acquire;
 using ptx::named_bar_sync;
 using ptx::pair_rows;
 using ptx::red_release_add;
-
-// silu with the fast divide: H is rounded to bf16 right after
-__device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __expf(-z)); }
 
 // A store that asks L2 to keep the line (the slot rows are read back by the combine right
 // after this launch, while the weights stream through L2 with evict-first)
@@ -881,19 +879,26 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
           for (int s = 0; s < 2; ++s)
 #pragma unroll
             for (int j = 0; j < 16; ++j) asm volatile("" : "+f"(v[s][j]));   // only after the wait
-          float h[2][8];
+          float h[16], up[16];
 #pragma unroll
           for (int s = 0; s < 2; ++s)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const float other =
                   __shfl_xor_sync(0xffffffffu, is_gate ? v[s][8 + j] : v[s][j], kGateRows);
-              h[s][j] = silu_f(is_gate ? v[s][j] : other) * (is_gate ? other : v[s][8 + j]);
+              h[8 * s + j] = is_gate ? v[s][j] : other;
+              up[8 * s + j] = is_gate ? other : v[s][8 + j];
             }
+          silu_all(h);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) h[j] *= up[j];
 #pragma unroll
           for (int s = 0; s < 2; ++s) {
+            float hs[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) hs[j] = h[8 * s + j];
             uint32_t w[4];
-            pair_rows(h[s], w);
+            pair_rows(hs, w);
             const int t0 = (s == 0 ? c0 : c0 + 32) + (is_gate ? 0 : 8) + 4 * odd;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
