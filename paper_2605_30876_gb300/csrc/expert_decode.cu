@@ -559,14 +559,19 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     bool ok = true, first = half == 0;
     // nstages stages of kboxes K boxes each; A's K boxes abox bytes apart, its groups of eight
     // rows sbo, M = mrows
+    // in_turn: the issuers take the K boxes of a stage in turn instead of by halves. Above 48
+    // tokens 32-row units do as 64-row units must (two boxes a stage): each part then sums the same
+    // K boxes in the same order, and a token's output has the same bits at both heights. (Up to 48
+    // tokens the parts are halves of a stage, as the outputs there have always been summed.)
     auto run = [&](int nstages, int kboxes, int abox, uint32_t sbo, uint32_t mrows, int value,
-                   bool gu) {
+                   bool gu, bool in_turn) {
       const uint32_t n_mma = (uint32_t)((p.T + 15) & ~15);
       const uint32_t idesc = ptx::idesc_bf16(mrows, n_mma);
       if (!wait(&acc_empty[acc], acc_phase ^ 1u, value)) { ok = false; return; }
       ptx::tc_fence_after();
       const uint32_t d0 = tmem_base + (uint32_t)((half * p.n_acc + acc) * p.n_pad);
-      const int kb0 = half * (kboxes / 2), kb1 = kb0 + kboxes / 2;
+      const int kb0 = in_turn ? half : half * (kboxes / 2), kbs = in_turn ? 2 : 1;
+      const int kb1 = kb0 + kboxes / 2 * kbs;
       for (int c = 0; c < nstages; ++c) {
         if (!wait(&full[stage], phase, value)) { ok = false; return; }
         if (gu && first && c == 0) ED_AT(2);
@@ -577,7 +582,7 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
         ptx::tc_fence_after();
         const uint32_t a0 = ptx::smem_addr(slot_a(stage));
         const uint32_t b0 = ptx::smem_addr(slot_b(stage));
-        for (int kb = kb0; kb < kb1; ++kb)
+        for (int kb = kb0; kb < kb1; kb += kbs)
 #pragma unroll
           for (int kk = 0; kk < kTileK / 16; ++kk)
             ptx::mma_bf16(d0, ptx::sdesc_k_sw128(a0 + kb * abox + kk * 32, sbo),
@@ -593,14 +598,15 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       int gi, m;
       gu_unit(u, gi, m);
       // all T token columns: the B box is x (rows >= T are zeros)
-      run(kc, kbg, kGateRows * 128, (uint32_t)(kbg * kGateRows * 128), (uint32_t)(2 * hg), u, true);
+      run(kc, kbg, kGateRows * 128, (uint32_t)(kbg * kGateRows * 128), (uint32_t)(2 * hg), u, true,
+          p.n_pad > 48);
       if (first) ED_AT(3);
       first = false;
     }
     first = half == 0;
     for (int v = v0; v < ND && ok; v += nb) {
       const Grp g = group_w(v / ndn);
-      run(g.Ig / kStageK, kKB, kABox, 1024u, (uint32_t)kTileM, v, false);
+      run(g.Ig / kStageK, kKB, kABox, 1024u, (uint32_t)kTileM, v, false, false);
       if (first) ED_AT(7);
       first = false;
     }
