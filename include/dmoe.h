@@ -124,8 +124,12 @@ dmoe_status dmoe_router(const dmoe_layer_desc* desc, const void* x, const float*
  * writes that split into the workspace and remembers on the host that the workspace holds
  * it for this w_r pointer; router and layer calls on the workspace with the same w_r then
  * skip the split. Call it again after changing W_r in place. A call with another w_r
- * splits that one, and the workspace then no longer holds this one's split. A no-op for
- * shapes whose router reads W_r directly.
+ * splits that one, and the workspace then no longer holds this one's split. Calls with
+ * another desc may share the workspace: the place of the split follows from the desc, so
+ * they split for themselves, and one that may write over this split ends its preparation
+ * (the next call splits again). A captured call keeps what it skipped: replay it only
+ * while the preparation it was captured with holds. A no-op for shapes whose router reads
+ * W_r directly.
  *   w_r      fp32 [d, E]     device, router weight (read)
  *   workspace                as for dmoe_router; stream: the CUDA stream of the split */
 dmoe_status dmoe_router_prepare(const dmoe_layer_desc* desc, const float* w_r, void* workspace,

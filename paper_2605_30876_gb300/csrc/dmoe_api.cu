@@ -13,17 +13,24 @@ namespace dmoe {
 namespace {
 thread_local char g_last_error[256] = "";
 
-// Workspaces whose W_r parts were written by dmoe_router_prepare, with the W_r they hold.
+// Workspaces whose W_r parts were written by dmoe_router_prepare: the W_r they hold, and where and
+// in what shape (both follow from the desc: calls with several descs may share a workspace).
+struct PreparedParts {
+  const void* w_r;
+  size_t offset;
+  int d, E;
+  bool at(size_t o, int dd, int ee) const { return offset == o && d == dd && E == ee; }
+};
 std::mutex g_prep_mu;
-std::unordered_map<const void*, const void*> g_prep;
+std::unordered_map<const void*, PreparedParts> g_prep;
 
-// Does `ws` hold the parts of `w_r`? If not, the split this call makes writes w_r's parts
-// there, so an earlier preparation of the workspace no longer holds.
-bool parts_prepared(const void* ws, const void* w_r) {
+// Does `ws` hold the parts of `w_r` where this call's layout has them? If it holds another W_r's
+// there, the split this call makes overwrites it, so the preparation no longer holds.
+bool parts_prepared(const void* ws, const void* w_r, size_t offset, int d, int E) {
   std::lock_guard<std::mutex> lock(g_prep_mu);
   auto it = g_prep.find(ws);
-  if (it == g_prep.end()) return false;
-  if (it->second == w_r) return true;
+  if (it == g_prep.end() || !it->second.at(offset, d, E)) return false;
+  if (it->second.w_r == w_r) return true;
   g_prep.erase(it);
   return false;
 }
@@ -74,6 +81,12 @@ void prof_end(int kernel, cudaStream_t s) {
   if (g_prof[kernel].end != nullptr) prof_record(g_prof[kernel].end, s);
 }
 bool prof_serial(int kernel) { return g_prof[kernel].begin != nullptr; }
+
+void drop_parts_below(const void* ws, size_t end) {
+  std::lock_guard<std::mutex> lock(g_prep_mu);
+  auto it = g_prep.find(ws);
+  if (it != g_prep.end() && it->second.offset < end) g_prep.erase(it);
+}
 
 void set_last_error(cudaError_t e) {
   snprintf(g_last_error, sizeof(g_last_error), "%s: %s", cudaGetErrorName(e),
@@ -177,6 +190,14 @@ dmoe_status check_ws(const dmoe_layer_desc* d, void* ws, size_t ws_bytes, Worksp
   *plan = plan_workspace(*d);
   if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return DMOE_ERR_INVALID_ARG;
   if (ws_bytes < plan->total) return DMOE_ERR_WORKSPACE;
+  // A call whose layout has its own regions where the workspace's prepared parts are may write
+  // over them: they are not taken for prepared after it. (With the same parts at the same place
+  // the layout's other regions leave them alone.)
+  std::lock_guard<std::mutex> lock(g_prep_mu);
+  auto it = g_prep.find(ws);
+  if (it != g_prep.end() && it->second.offset < plan->total &&
+      !(plan->w_parts_bytes > 0 && it->second.at(plan->w_parts, d->d_model, d->n_experts)))
+    g_prep.erase(it);
   return DMOE_OK;
 }
 
@@ -238,7 +259,8 @@ dmoe_status run_router(const dmoe_layer_desc* desc, const void* x, const float* 
   a.err = at<DevErrRecord>(ws, plan.err);
   a.shared_pf = shared_pf;
   a.w_parts = plan.w_parts_bytes > 0 ? at<__nv_bfloat16>(ws, plan.w_parts) : nullptr;
-  a.parts_ready = a.w_parts != nullptr && parts_prepared(ws, w_r);
+  a.parts_ready = a.w_parts != nullptr &&
+                  parts_prepared(ws, w_r, plan.w_parts, desc->d_model, desc->n_experts);
   a.tc_splits = plan.tc_splits;
   a.tc_part = plan.tc_splits > 0 ? at<float>(ws, plan.tc_part) : nullptr;
   return cuda_status(launch_router(a, dsp, at<int32_t>(ws, plan.tickets), s));
@@ -374,7 +396,7 @@ dmoe_status dmoe_router_prepare(const dmoe_layer_desc* desc, const float* w_r, v
                                              static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_status(e);
   std::lock_guard<std::mutex> lock(g_prep_mu);
-  g_prep[workspace] = w_r;
+  g_prep[workspace] = PreparedParts{w_r, plan.w_parts, desc->d_model, desc->n_experts};
   return DMOE_OK;
 }
 

@@ -373,6 +373,9 @@ inline cudaError_t max_shared_carveout(F* kernel, std::atomic<uint32_t>& done) {
 }
 
 // host helpers
+// The bytes of `ws` before `end` are written by a call that has no workspace layout of its own
+// there: parts that dmoe_router_prepare wrote below `end` are not taken for prepared any more.
+void drop_parts_below(const void* ws, size_t end);
 int device_sm_count();
 void set_last_error(cudaError_t e);
 void set_last_error_text(const char* msg);

@@ -86,6 +86,7 @@ extern "C" dmoe_status dmoe_router_no_alloc(const dmoe_layer_desc* desc, const v
     set_last_error(e);
     return DMOE_ERR_CUDA;
   }
+  drop_parts_below(scratch, need);   // (the array may have been given to a call as a workspace)
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // The fault record is not cleared here: as in a caller workspace, a recorded fault stays
   // until dmoe_router_no_alloc_device_error reads it (the array starts zero-filled when the
