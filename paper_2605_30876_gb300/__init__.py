@@ -267,7 +267,7 @@ def dmoe_no_alloc_scratch() -> Tuple[int, int]:
 
 
 def dmoe_set_debug_hold(workspace, hold: int, stream=None) -> None:
-    """Diagnostic: makes the decode-size expert launch's bounded waits run out while
+    """Diagnostic: makes the expert launch's bounded waits run out while
     `hold` is nonzero (see include/dmoe.h); cleared by dmoe_get_device_error."""
     _check(_lib.dmoe_set_debug_hold(_ptr(workspace, torch.uint8, "workspace"), int(hold),
                                     _stream(stream)), "dmoe_set_debug_hold")

@@ -515,13 +515,15 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   };
 
   // The cluster's i-th unit for a role of this CTA: a thread, or (warp_wide) a warp, all lanes
-  // of which read it. The entry is free again once all roles have read it.
+  // of which read it. The entry is free again once all roles have read it. A wait that failed gives
+  // an end, and the entry stays taken: another role may still have to read what it held before.
   auto unit_at = [&](int i, bool warp_wide) -> Unit {
     const int e = i % kQueue;
-    const bool got = wait(&d_full[e], (uint32_t)(i / kQueue) & 1u, i);
+    bool got = wait(&d_full[e], (uint32_t)(i / kQueue) & 1u, i);
+    if (warp_wide) got = __all_sync(0xffffffffu, got);
     const Unit un = unpack(got ? s_desc[e] : make_int2(-1, 0));
     if (warp_wide) __syncwarp();
-    if (!warp_wide || lane == 0) ptx::mbar_arrive(&d_empty[e]);
+    if (got && (!warp_wide || lane == 0)) ptx::mbar_arrive(&d_empty[e]);
     return un;
   };
   // Steps (K = 128) are counted over all units of the cluster; one commit per step reports to
@@ -532,17 +534,10 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   auto step_done = [&](int t, int value) -> bool {
     return wait(&progress[t % kProgress], (uint32_t)(t / kProgress) & 1u, value);
   };
-  // after a failed wait: lets this producer's copies in flight land before the CTA exits (they
-  // complete on the first CTA's barriers, together with the other CTA's: a slot that one left
-  // unfilled runs the bounded wait out)
-  auto drain_copies = [&](uint64_t* full, int stages, int st, uint32_t ph, int issued) {
-    for (int i = issued < stages ? issued : stages; i > 0; --i) {
-      if (--st < 0) { st = stages - 1; ph ^= 1u; }
-      const uint64_t t0 = ptx::globaltimer_ns();
-      while ((rank != 0 || !ptx::mbar_try_wait(&full[st], ph)) &&
-             ptx::globaltimer_ns() - t0 < kWaitTimeoutNs / 10) {
-      }
-    }
+  // A producer leaves only once the MMAs of its last step are done, which its copies came before;
+  // if they do not come to be done, the abort flag is set and the CTA stays a while (see the end).
+  auto landed = [&](int steps) {
+    if (steps > 0) step_done(steps - 1, -1);
   };
 
   if (warp == 0) {
@@ -554,7 +549,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       const uint64_t pol_norm = ptx::policy_evict_normal();   // ... or by several
       const uint32_t full0 = ptx::peer_smem(a_full, 0);
       int stage = 0, chunk = 0;
-      uint32_t phase = 0;
       bool ok = true;
       for (int i = 0; ok; ++i) {
         const Unit un = unit_at(i, false);
@@ -591,7 +585,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
                                     bar + 8u * (uint32_t)(j / 4), 0, 0, c,
                                     arow / 8 + (j >> 1) * (kGateRows / 8), pol_w);
           }
-          if (++stage == a_stages) { stage = 0; phase ^= 1u; }
+          if (++stage == a_stages) stage = 0;
           if (rank == 0 && c == kc / 2) {
             if (i == 0) {
               if (!spec) pdl_wait();   // the counter is zero from here on
@@ -606,7 +600,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         }
         if (TRU(i) < 8) DMOE_TRACE_AT(4 + 6 * TRU(i));
       }
-      if (!ok) drain_copies(a_full, a_stages, stage, phase, chunk);
+      landed(chunk >> 1);
     }
   } else if (warp == kRowWarp) {
     // ================= TMA producer of the token rows (x or H; lane i issues the i-th box of a
@@ -615,7 +609,6 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     const uint64_t pol_x = ptx::policy_evict_last();    // activations: re-read by tiles
     const uint32_t full0 = ptx::peer_smem(b_full, 0);
     int stage = 0, issued = 0;
-    uint32_t phase = 0;
     int step0 = 0;          // the unit's first step
     if (!spec) pdl_wait();   // the rows in dispatch order are complete from here on
     int last = 0;           // lane s: the last step that reads what slot s holds
@@ -685,21 +678,27 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         }
         if (lane == stage) last = step0 + (min(c + kpb, kc) - 1) / 2;
         ++issued;
-        if (++stage == b_stages) { stage = 0; phase ^= 1u; }
+        if (++stage == b_stages) stage = 0;
       }
       step0 += kc / 2;
     }
-    if (!ok && lane == 0) drain_copies(b_full, b_stages, stage, phase, issued);
+    if (lane == 0) landed(step0);
   } else if (warp == kPlanWarp) {
     // ================= the units, decoded one or more ahead of their use, and the readiness of
     // their token rows (a poll is an L2 round trip, 1 us or more while weights stream)
     if (lane == 0) {
       const uint32_t q_empty0 = ptx::peer_smem(q_empty, 0);
+      // diagnostic (normally 0): every down unit waits for this many more gate/up tiles than its
+      // group has, so that its bounded wait runs out (read once the first unit is handed on: at
+      // the start of the kernel it held every launch up by 0.6 to 1.1 us)
+      int hold = 0;
       for (int i = 0;; ++i) {
         int u = cl;
         if (i > 0) {
           const int q = (i - 1) % kQueue;
-          u = wait(&q_full[q], (uint32_t)((i - 1) / kQueue) & 1u, i) ? s_queue[q] : units;
+          // (a wait that failed: the other roles leave by the abort flag)
+          if (!wait(&q_full[q], (uint32_t)((i - 1) / kQueue) & 1u, i)) break;
+          u = s_queue[q];
           ptx::mbar_arrive_expect_tx(&q_full[q], 4);   // the entry's next unit
           ptx::mbar_arrive_pair(q_empty0 + 8u * (uint32_t)q);
         }
@@ -708,12 +707,13 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         if (i >= kQueue && !wait(&d_empty[e], ((uint32_t)(i / kQueue) & 1u) ^ 1u, i)) break;
         s_desc[e] = d;
         ptx::mbar_arrive(&d_full[e]);
+        if (i == 0) hold = *reinterpret_cast<volatile int32_t*>(&p.err->hold);
         const Unit un = unpack(d);
         if (un.end) break;
         if (!un.gu) {
           if (!spec) pdl_wait();   // the counters are zeroed from here on
           const int32_t* flag = p.h_ready + un.g * p.ntiles + un.n;
-          const int need = (un.shared ? p.Is : p.I) / 64;
+          const int need = (un.shared ? p.Is : p.I) / 64 + hold;
           bool ok = true;
           if (ld_acquire(flag) < need) {
             const uint64_t t0 = ptx::globaltimer_ns();
@@ -966,6 +966,13 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   if (warp == 1) {
     __syncwarp();
     ptx::tmem_dealloc2(tmem_base, p.tmem_cols);
+  }
+  // After a wait that failed, copies into this CTA's shared memory and stores and arrivals from the
+  // other CTA may not have been waited for. Nothing new is issued any more (the barrier above): the
+  // CTA stays until they have long landed (they take microseconds).
+  if (*s_abort) {
+    const uint64_t t0 = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - t0 < kWaitTimeoutNs / 10) __nanosleep(1000);
   }
 }
 

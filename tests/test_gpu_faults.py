@@ -1,9 +1,9 @@
 """Failure detection without a GPU fault: a bounded device-side wait that runs out.
 
-dmoe_set_debug_hold makes every down tile of the decode-size expert launch wait for more
-gate/up tiles than its group has (a count nothing will reach). The wait gives up after its
-1 s limit: the kernel records DMOE_ERR_TIMEOUT in the workspace, lets its in-flight copies
-land, frees its tensor memory and exits; no trap, no unbounded wait. dmoe_get_device_error
+dmoe_set_debug_hold makes every down tile of the expert launch (decode size, and the general
+one: pairs of CTAs) wait for more gate/up tiles than its group has (a count nothing will
+reach). The wait gives up after its 1 s limit: the kernel records DMOE_ERR_TIMEOUT in the
+workspace, lets its in-flight copies land, frees its tensor memory and exits; no trap, no unbounded wait. dmoe_get_device_error
 reports the timeout and clears it (with the hold), and the next call on the same workspace
 is a normal, parity-checked forward."""
 import time
@@ -20,7 +20,17 @@ TIMEOUT = 6          # DMOE_ERR_TIMEOUT
 ERR_TIMEOUT = 1      # the record's code for a bounded wait that ran out
 
 
-@pytest.mark.parametrize("shape", [TINY, TINY.with_(mode=ROUTE_TOKEN)], ids=["block", "token"])
+GENERAL = TINY.with_(block_size=32, n_blocks=5, d_ff_shared=128)
+SHAPES = {
+    "block": TINY, "token": TINY.with_(mode=ROUTE_TOKEN),
+    "general_block": GENERAL, "general_p06": GENERAL.with_(top_p=0.6),
+    "general_token": GENERAL.with_(mode=ROUTE_TOKEN),
+    # more units than clusters, more steps than ring slots, more than one token tile
+    "general_block_many": GENERAL.with_(n_blocks=20, d_model=640, d_ff=512, top_k=8),
+}
+
+
+@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES)
 def test_bounded_wait_times_out_and_the_workspace_recovers(shape):
     m = P.dm()
     from paper_2605_30876_gb300.layer import MoELayer
