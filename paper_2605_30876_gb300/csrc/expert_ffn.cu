@@ -544,14 +544,17 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
     // ================= TMA producer of the weights: waits for ring slots only, so the weights
     // of the next unit follow those of the last without a gap. The bytes of both CTAs
     // complete on the first CTA's barriers, where its producers expect them.
-    if (lane == 0) {
+    // kFar: the whole warp, lane j issues the j-th of a step's eight boxes.
+    if (kFar || lane == 0) {
+      // a wait's result for every lane that takes part
+      auto agreed = [&](bool v) { return kFar ? __all_sync(0xffffffffu, v) != 0 : v; };
       const uint64_t pol_first = ptx::policy_evict_first();   // weights read by one tile
       const uint64_t pol_norm = ptx::policy_evict_normal();   // ... or by several
       const uint32_t full0 = ptx::peer_smem(a_full, 0);
       int stage = 0, chunk = 0;
       bool ok = true;
       for (int i = 0; ok; ++i) {
-        const Unit un = unit_at(i, false);
+        const Unit un = unit_at(i, kFar);
         if (un.end) break;
         const bool shared = un.shared;
         const uint64_t pol_w = g_cnt[un.g] > p.n_max ? pol_norm : pol_first;
@@ -559,7 +562,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         // the next unit: the first CTA asks for it now and enters it for both CTAs once half
         // of this unit's loads are issued
         int next = units;
-        if (rank == 0 && i > 0) next = ncl + atomicAdd(p.next_unit, 1);
+        if (rank == 0 && lane == 0 && i > 0) next = ncl + atomicAdd(p.next_unit, 1);
         const int kc = (un.gu ? p.d : (shared ? p.Is : p.I)) / kTileK;
         // (d % 256 = 128: the last down unit's second half reads the rows that follow and
         // stores nothing)
@@ -570,32 +573,34 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
         const CUtensorMap* m01 = shared ? &tm.sgu : &tm.gu;
         for (int c = 0; c < kc; ++c, ++chunk) {
           // the slot's last K step was chunk - a_stages
-          if (chunk >= a_stages && !step_done((chunk - a_stages) >> 1, i)) { ok = false; break; }
-          if (rank == 0) ptx::mbar_arrive_expect_tx(&a_full[stage], kCluster * kATileBytes);
+          if (chunk >= a_stages && !agreed(step_done((chunk - a_stages) >> 1, i))) {
+            ok = false;
+            break;
+          }
+          if (rank == 0 && lane == 0)
+            ptx::mbar_arrive_expect_tx(&a_full[stage], kCluster * kATileBytes);
           uint8_t* dst = smem + off_a + stage * kATileBytes;
           const uint32_t bar = full0 + 8u * (uint32_t)stage;
           if (!un.gu) {
-            ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow, pol_w);
+            if (lane == 0) ptx::tma_load_2d_pair(dst, m0, bar, c * kTileK, arow, pol_w);
           } else if (!kFar) {
             ptx::tma_load_4d_pair(dst, m01, bar, c * kTileK, 0, 0, arow / kGateRows, pol_w);
-          } else if ((c & 1) == 0) {   // two slots at once (their number is even)
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              ptx::tma_load_4d_pair(dst + j * 2 * kGateRows * 128, (j & 1) ? m1 : m0,
-                                    bar + 8u * (uint32_t)(j / 4), 0, 0, c,
-                                    arow / 8 + (j >> 1) * (kGateRows / 8), pol_w);
+          } else if ((c & 1) == 0 && lane < 8) {   // two slots at once (their number is even)
+            ptx::tma_load_4d_pair(dst + lane * 2 * kGateRows * 128, (lane & 1) ? m1 : m0,
+                                  bar + 8u * (uint32_t)(lane / 4), 0, 0, c,
+                                  arow / 8 + (lane >> 1) * (kGateRows / 8), pol_w);
           }
           if (++stage == a_stages) stage = 0;
           if (rank == 0 && c == kc / 2) {
             if (i == 0) {
               if (!spec) pdl_wait();   // the counter is zero from here on
-              next = ncl + atomicAdd(p.next_unit, 1);
+              if (lane == 0) next = ncl + atomicAdd(p.next_unit, 1);
             }
-            if (i >= kQueue && !wait(&q_empty[i % kQueue], ((i / kQueue) & 1) ^ 1, i)) {
+            if (i >= kQueue && !agreed(wait(&q_empty[i % kQueue], ((i / kQueue) & 1) ^ 1, i))) {
               ok = false;
               break;
             }
-            enter_unit(i + 1, next);
+            if (lane == 0) enter_unit(i + 1, next);
           }
         }
         if (TRU(i) < 8) DMOE_TRACE_AT(4 + 6 * TRU(i));
