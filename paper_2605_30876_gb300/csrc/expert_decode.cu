@@ -97,8 +97,7 @@ struct DParams {
   int h32_ok;                // 32-row gate/up units allowed (d % 256 == 0, >= 3 slots fit)
   int has_shared;
   int gu_box, sgu_box;       // gate and up rows come in one box (DMaps::gu ..): 1: gate first, 2:
-                             // up first (routed experts, shared expert)
-  int far;                   // ... or in boxes of their own, gate first (DMaps::wg ..), in both
+                             // up first (routed experts, shared expert); 0 in the kFar form
   int n_acc;                 // TMEM accumulators of n_pad columns
   uint32_t tmem_cols;
 };
@@ -138,29 +137,31 @@ __device__ __forceinline__ float silu_f(float z) { return __fdividef(z, 1.f + __
 
 // One gate/up stage's weights: hg (32 or 64) rows of W_gate and the same rows of W_up from row
 // arow, some of each in turn (gate_rows), over the 64-column K boxes from kb on (32 KB): each 8
-// rows over all K boxes of the stage, 1 KB a box. Tensors too far apart for one map (allocations
-// in two address ranges) take 8 copies of 4 KB (98 unique experts, I = 384: one map 87 us, 32
-// copies of 1 KB 150, 16 of 2 KB 113).
-__device__ __forceinline__ void load_gate_up(const DMaps& tm, const DParams& p, uint8_t* dst,
-                                             uint64_t* bar, bool shared, bool h32, int arow, int kb,
+// rows over all K boxes of the stage, 1 KB a box. kFar: tensors too far apart for one map
+// (allocations in two address ranges) take 8 copies of 4 KB, one each from lanes 0 to 7 of the
+// calling warp (98 unique experts, I = 384: one map 87 us, 32 copies of 1 KB 150, 16 of 2 KB 113).
+template <bool kFar>
+__device__ __forceinline__ void load_gate_up(const DMaps& tm, uint8_t* dst, uint64_t* bar,
+                                             bool shared, bool h32, int arow, int kb,
                                              uint64_t pol) {
-  if (!p.far) {
+  if (!kFar) {
     const CUtensorMap* m = shared ? (h32 ? &tm.sgu32 : &tm.sgu) : (h32 ? &tm.gu32 : &tm.gu);
     ptx::tma_load_5d(dst, m, bar, 0, 0, kb, 0, arow / kGateRows, pol);
     return;
   }
+  const int j = threadIdx.x & 31;
+  if (j >= 8) return;
   const CUtensorMap* mg = shared ? (h32 ? &tm.sg32 : &tm.sg) : (h32 ? &tm.wg32 : &tm.wg);
   const CUtensorMap* mu = shared ? (h32 ? &tm.su32 : &tm.su) : (h32 ? &tm.wu32 : &tm.wu);
-  for (int j = 0; j < 4; ++j, dst += kAStage / 4) {
-    const int r8 = arow / 8 + (h32 ? j : 2 * j);
-    ptx::tma_load_4d(dst, mg, bar, 0, 0, kb, r8, pol);
-    ptx::tma_load_4d(dst + kAStage / 8, mu, bar, 0, 0, kb, r8, pol);
-  }
+  ptx::tma_load_4d(dst + j * (kAStage / 8), (j & 1) ? mu : mg, bar, 0, 0, kb,
+                   arow / 8 + (j >> 1) * (h32 ? 1 : 2), pol);
 }
 
 // kMask: the coresets are published as masks (DParams::spec_mask), compiled separately so
-// that the launch on ids carries none of that code
-template <bool kMask>
+// that the launch on ids carries none of that code; so is kFar: gate and up weights in boxes of
+// their own (DMaps::wg ..), issued by eight lanes of the producer's warp. (As a branch in the one
+// kernel that form cost every launch 0.1 to 0.3 us.)
+template <bool kMask, bool kFar>
 __global__ void __launch_bounds__(kThr, 1)
 moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -300,8 +301,8 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       }
       if (lane == 0) *s_u = bad ? -1 : u_all;
       __syncwarp();
-      if (lane == 0 && !bad) {
-        // This lane is the producer: the first ring slots of its first gate/up unit are
+      if ((kFar || lane == 0) && !bad) {
+        // This lane (kFar: warp) is the producer: the first ring slots of its first gate/up unit are
         // filled now, before the CTA barrier and the unit bookkeeping below (the same copies
         // the producer loop would make; fresh ring slots need no wait).
         const bool h32e = h32_ok && 2 * (ngu64_s + u_all * ngu64_r) <= nb;
@@ -318,10 +319,12 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
           early = Se < kce ? Se : kce;
           ED_AT(28);
           for (int c = 0; c < early; ++c) {
-            ptx::mbar_arrive_expect_tx(&full[c], kAStage + kbge * bbox);
             uint8_t* a_dst = smem + c * slote;
-            load_gate_up(tm, p, a_dst, &full[c], sh, h32e, arow, c * kbge, pw);
-            ptx::tma_load_3d(a_dst + kAStage, h32e ? &tm.x32 : &tm.x, &full[c], 0, 0, c * kbge, px);
+            if (lane == 0) ptx::mbar_arrive_expect_tx(&full[c], kAStage + kbge * bbox);
+            load_gate_up<kFar>(tm, a_dst, &full[c], sh, h32e, arow, c * kbge, pw);
+            if (lane == 0)
+              ptx::tma_load_3d(a_dst + kAStage, h32e ? &tm.x32 : &tm.x, &full[c], 0, 0, c * kbge,
+                               px);
           }
         }
       }
@@ -451,8 +454,9 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
   };
   const int kc = h32 ? kc32 : kc64;   // stages of one gate/up tile
 
-  if (warp == 0 && lane == 0) {
-    // ================= TMA producer
+  if (warp == 0 && (kFar || lane == 0)) {
+    // ================= TMA producer (kFar: the whole warp waits, lane 0 issues what is one copy)
+    auto agreed = [&](bool v) { return kFar ? __all_sync(0xffffffffu, v) != 0 : v; };
     const uint64_t pol_w = ptx::policy_evict_first();   // weights: streamed once
     const uint64_t pol_x = ptx::policy_evict_last();    // x and H: re-read by many tiles
     ED_AT(31);
@@ -468,12 +472,14 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       const int arow = (g.shared ? 0 : g.e * p.I) + m * hg;
       if (first) ED_SET(10, u);
       for (int c = first ? early : 0; c < kc; ++c) {
-        if (!wait(&empty[stage], phase ^ 1u, u)) { ok = false; break; }
+        if (!agreed(wait(&empty[stage], phase ^ 1u, u))) { ok = false; break; }
         if (first && c == 0) ED_AT(28);
         if (first && c == kc - 1) ED_AT(29);
-        ptx::mbar_arrive_expect_tx(&full[stage], kAStage + kbg * bbox);
-        load_gate_up(tm, p, slot_a(stage), &full[stage], g.shared, h32, arow, c * kbg, pol_w);
-        ptx::tma_load_3d(slot_b(stage), h32 ? &tm.x32 : &tm.x, &full[stage], 0, 0, c * kbg, pol_x);
+        if (lane == 0) ptx::mbar_arrive_expect_tx(&full[stage], kAStage + kbg * bbox);
+        load_gate_up<kFar>(tm, slot_a(stage), &full[stage], g.shared, h32, arow, c * kbg, pol_w);
+        if (lane == 0)
+          ptx::tma_load_3d(slot_b(stage), h32 ? &tm.x32 : &tm.x, &full[stage], 0, 0, c * kbg,
+                           pol_x);
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -492,16 +498,18 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
       // weights first: they do not depend on the gate/up phase
       int done = 0;
       for (int c = 0; c < pre; ++c, ++done) {
-        if (!wait(&empty[stage], phase ^ 1u, v)) { ok = false; break; }
-        ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
-        ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
+        if (!agreed(wait(&empty[stage], phase ^ 1u, v))) { ok = false; break; }
+        if (lane == 0) {
+          ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
+          ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
+        }
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
       if (first) ED_AT(5);
       // then the H rows, once every gate/up tile of the group is published
       const int target = g.Ig / hg + hold;
-      if (ok && ld_acquire(p.h_ready + gi) < target) {
+      if (ok && lane == 0 && ld_acquire(p.h_ready + gi) < target) {
         const uint64_t t0 = ptx::globaltimer_ns();
         while (ld_acquire(p.h_ready + gi) < target) {
           if (*s_abort) { ok = false; break; }
@@ -513,11 +521,13 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
           }
         }
       }
+      ok = agreed(ok);
       fence_proxy_async_global();
       if (first) ED_AT(6);
       {
         int st = st0;
         for (int c = 0; c < done; ++c) {
+          if (lane != 0) break;   // (kFar)
           if (ok) {
             ptx::tma_load_3d(slot_b(st), &tm.h, &full[st], 0, gi * p.n_pad, c * kKB, pol_x);
           } else {
@@ -528,10 +538,12 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
         }
       }
       for (int c = pre; c < ndk && ok; ++c) {
-        if (!wait(&empty[stage], phase ^ 1u, v)) { ok = false; break; }
-        ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
-        ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
-        ptx::tma_load_3d(slot_b(stage), &tm.h, &full[stage], 0, gi * p.n_pad, c * kKB, pol_x);
+        if (!agreed(wait(&empty[stage], phase ^ 1u, v))) { ok = false; break; }
+        if (lane == 0) {
+          ptx::mbar_arrive_expect_tx(&full[stage], kAStage + bstage);
+          ptx::tma_load_3d(slot_a(stage), md, &full[stage], 0, arow, c * kKB, pol_w);
+          ptx::tma_load_3d(slot_b(stage), &tm.h, &full[stage], 0, gi * p.n_pad, c * kKB, pol_x);
+        }
         ++issued;
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
@@ -626,10 +638,10 @@ moe_decode_kernel(const __grid_constant__ DMaps tm, const __grid_constant__ DPar
     // turn (16 for M = 128 from tensors far apart), so the up row of a gate lane l is in lane
     // l + 8 (16) of the same warp
     const bool g_act = hg == 64 || lane < 16;
-    const int gate_rows = p.far && hg == 64 ? 16 : kGateRows;
+    const int gate_rows = kFar && hg == 64 ? 16 : kGateRows;
     // row of the tile
     const int rr = hg != 64 ? 8 * q + (lane & 7)
-                            : 16 * q + (p.far ? lane & 15 : 8 * (lane >> 4) + (lane & 7));
+                            : 16 * q + (kFar ? lane & 15 : 8 * (lane >> 4) + (lane & 7));
     const int n_mma = (p.T + 15) & ~15;
     const uint32_t part1 = (uint32_t)(p.n_acc * p.n_pad);   // column offset of part 1
     // 16 columns of an accumulator: the sum of its two parts
@@ -958,8 +970,8 @@ cudaError_t launch_experts_decode(const ExpertArgs& a, cudaStream_t s) {
       p.sgu_box = make_map_two(&m.sgu32, a.ws_gate, a.ws_up, (uint64_t)a.Is, a.d, 32, kTileM / 32);
   }
   // tensors too far apart for one map: all of them in boxes of their own
-  p.far = p.gu_box == 0 || (has_shared && p.sgu_box == 0) ? 1 : 0;
-  if (p.far) {
+  const bool far = p.gu_box == 0 || (has_shared && p.sgu_box == 0);
+  if (far) {
     p.gu_box = p.sgu_box = 0;
     auto apart = [&](CUtensorMap* m64, CUtensorMap* m32, const void* w, uint64_t rows) {
       return make_map_far(m64, w, rows, a.d, 16, 2) &&
@@ -1001,12 +1013,12 @@ cudaError_t launch_experts_decode(const ExpertArgs& a, cudaStream_t s) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (dev >= 31 || !(attr_dev_mask & (1 << dev))) {
-      cudaError_t e = cudaFuncSetAttribute(moe_decode_kernel<false>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           max_smem_optin());
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(moe_decode_kernel<true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem_optin());
+      cudaError_t e = cudaSuccess;
+      for (auto* kernel : {moe_decode_kernel<false, false>, moe_decode_kernel<true, false>,
+                           moe_decode_kernel<false, true>, moe_decode_kernel<true, true>})
+        if (e == cudaSuccess)
+          e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   max_smem_optin());
       if (e != cudaSuccess) return e;
       if (dev < 31) attr_dev_mask |= 1 << dev;
     }
@@ -1017,11 +1029,10 @@ cudaError_t launch_experts_decode(const ExpertArgs& a, cudaStream_t s) {
   if (a.spec_words != nullptr && grid > 2 * kRouteClusterCtas) grid -= kRouteClusterCtas;
   if (grid > kMaxPersistentCtas) grid = kMaxPersistentCtas;
   prof_begin(DMOE_KERNEL_EXPERTS, s);
-  cudaError_t e =
-      p.spec_mask ? launch_ex(moe_decode_kernel<true>, dim3(grid), dim3(kThr), smem, s,
-                              !prof_serial(DMOE_KERNEL_EXPERTS), m, p)
-                  : launch_ex(moe_decode_kernel<false>, dim3(grid), dim3(kThr), smem, s,
-                              !prof_serial(DMOE_KERNEL_EXPERTS), m, p);
+  cudaError_t e = launch_ex(
+      far ? (p.spec_mask ? moe_decode_kernel<true, true> : moe_decode_kernel<false, true>)
+          : (p.spec_mask ? moe_decode_kernel<true, false> : moe_decode_kernel<false, false>),
+      dim3(grid), dim3(kThr), smem, s, !prof_serial(DMOE_KERNEL_EXPERTS), m, p);
   prof_end(DMOE_KERNEL_EXPERTS, s);
   if (e != cudaSuccess) return e;
   // the expert launch releases the combine at its end, after its wait for the routing
