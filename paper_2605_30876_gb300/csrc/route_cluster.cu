@@ -125,6 +125,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+template <bool kTopK>
 __global__ void __launch_bounds__(256, 1)
 route_cluster_kernel(const __grid_constant__ ClusterArgs f) {
   // 1024-B aligned: the swizzled x boxes take their swizzle phase from the address
@@ -449,11 +450,11 @@ route_cluster_kernel(const __grid_constant__ ClusterArgs f) {
       const int t0 = b * B;
       // block top-k: the coreset (k experts) is the routing of every token of the block; it
       // is published for the expert launch as soon as it is known
-      const int size = block_coreset_steps(
+      const int size = block_coreset_steps<kTopK>(
           E, kc, B, a.top_p, [&](int i, int e) { return sHat[(t0 + i) * kMaxExperts + e]; }, order,
           a.coreset != nullptr ? a.coreset + (size_t)b * E : nullptr,
           a.coreset_size != nullptr ? a.coreset_size + b : nullptr,
-          a.spec_words != nullptr && !a.spec_mask && a.top_p <= 0.f && kc == k
+          a.spec_words != nullptr && !a.spec_mask && kTopK && kc == k
               ? a.spec_words + (size_t)b * spec_words(k)
               : nullptr,
           sHat + (size_t)t0 * kMaxExperts, kMaxExperts);
@@ -640,9 +641,11 @@ cudaError_t launch_cluster_common(const RouterArgs& a, const DispatchArgs* dsp,
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 31 || !(mask & (1 << dev))) {
-    cudaError_t e = cudaFuncSetAttribute(route_cluster_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_max);
+    cudaError_t e = cudaSuccess;
+    for (auto* kernel : {route_cluster_kernel<false>, route_cluster_kernel<true>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem_max);
     if (e != cudaSuccess) return e;
     if (dev < 31) mask |= 1 << dev;
   }
@@ -650,7 +653,9 @@ cudaError_t launch_cluster_common(const RouterArgs& a, const DispatchArgs* dsp,
             logits_only ? (a.T + kClMaxTok - 1) / kClMaxTok : 1);
   // programmatic dependent launch: the set-up overlaps the previous kernel on the stream;
   // the kernel waits for it (griddepcontrol.wait) before it reads anything
-  return launch_cluster(route_cluster_kernel, grid, dim3(256), smem, s, kCl, true, f);
+  return launch_cluster(a.mode == DMOE_ROUTE_BLOCK && a.top_p > 0.f ? route_cluster_kernel<false>
+                                                                    : route_cluster_kernel<true>,
+                        grid, dim3(256), smem, s, kCl, true, f);
 }
 }  // namespace
 

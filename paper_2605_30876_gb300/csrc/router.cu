@@ -118,6 +118,7 @@ router_softmax_kernel(const float* __restrict__ part, int splits, const float* _
   KLOG(5, 1);
 }
 
+template <bool kTopK>
 __global__ void __launch_bounds__(256)
 block_route_kernel(const float* __restrict__ probs, const float* __restrict__ probs_hat,
                    int E, int kb, int k, int B, float top_p,
@@ -138,7 +139,7 @@ block_route_kernel(const float* __restrict__ probs, const float* __restrict__ pr
   pdl_launch_dependents();   // after the wait: a waiting dependent would share the SMs
   KLOG(6, 0);
   DMOE_STAMP(0);
-  block_route_cta(blockIdx.x, probs, probs_hat, E, kb, k, B, top_p, topk_idx, topk_gate, coreset,
+  block_route_cta<kTopK>(blockIdx.x, probs, probs_hat, E, kb, k, B, top_p, topk_idx, topk_gate, coreset,
                   coreset_size, spec);
   KLOG(6, 1);
 }
@@ -179,10 +180,12 @@ cudaError_t launch_router(const RouterArgs& a, const DispatchArgs* dsp, int32_t*
                   a.probs, a.probs_hat, a.topk_idx, a.topk_gate, a.T, a.E, a.kb, a.mode);
     if (e != cudaSuccess) return e;
     if (a.mode == DMOE_ROUTE_BLOCK) {
-      static std::atomic<uint32_t> carveout;
-      e = max_shared_carveout(block_route_kernel, carveout);
+      static std::atomic<uint32_t> carveout[2];
+      const bool topk = a.top_p <= 0.f;
+      auto* kernel = topk ? block_route_kernel<true> : block_route_kernel<false>;
+      e = max_shared_carveout(kernel, carveout[topk ? 1 : 0]);
       if (e != cudaSuccess) return e;
-      e = launch_ex(block_route_kernel, dim3(a.n_blocks), dim3(256), 0, s, true, a.probs,
+      e = launch_ex(kernel, dim3(a.n_blocks), dim3(256), 0, s, true, a.probs,
                     a.probs_hat, a.E, a.kb, a.k, a.B, a.top_p, a.topk_idx, a.topk_gate, a.coreset,
                     a.coreset_size, a.spec_words, a.ready_clear, a.n_ready_clear);
       if (e != cudaSuccess) return e;

@@ -223,7 +223,11 @@ __device__ inline void publish_coreset_mask(uint32_t* __restrict__ words, const 
 // taken by counting, without the normalisation. For p > 0 every nonzero S~ counts the nonzero
 // entries that beat it (larger, or equal with a lower id), all in parallel; p < 1 then adds
 // them in order up to the threshold. Needs blockDim.x == kMaxExperts.
-template <class HatFn>
+//
+// kTopK: p <= 0. A form of its own, as every launch runs this code once or a few times and fetches
+// it cold: with both rules in one kernel the layer of 16 tokens with p = 0.6 took 19.2 us (eight
+// in a graph), apart 18.4.
+template <bool kTopK, class HatFn>
 __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatFn hat, int* order,
                                           int32_t* __restrict__ coreset,
                                           int32_t* __restrict__ coreset_size,
@@ -280,7 +284,7 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     }
   }
   DMOE_STAMP(22);
-  if (top_p <= 0.f) {
+  if constexpr (kTopK) {
     // p <= 0 (block top-k): Top-P stops at the first entry and the floor extends the coreset
     // to the k best. S~ = S / sum(S) has the order of S (exactly so, where the fp32 division
     // would round two sums to one value), so the k best sums are taken directly, by counting:
@@ -558,7 +562,7 @@ __device__ inline void mask_topk_warps(int k, int B, int size, const int* order,
   }
 }
 
-template <class HatFn, class ProbFn, class OutFn>
+template <bool kTopK, class HatFn, class ProbFn, class OutFn>
 __device__ inline void block_route_steps(int E, int kb, int k, int B, float top_p, HatFn hat,
                                          ProbFn prob, OutFn out, int32_t* __restrict__ coreset,
                                          int32_t* __restrict__ coreset_size,
@@ -567,8 +571,8 @@ __device__ inline void block_route_steps(int E, int kb, int k, int B, float top_
   __shared__ int order[kMaxExperts];
   // block top-k (p <= 0, the coreset is every token's routing): published for the expert
   // launch as soon as it is known
-  const int size = block_coreset_steps(E, kb, B, top_p, hat, order, coreset, coreset_size,
-                                       top_p <= 0.f && kb == k ? spec : nullptr, hat_rows, E);
+  const int size = block_coreset_steps<kTopK>(E, kb, B, top_p, hat, order, coreset, coreset_size,
+                                              kb == k ? spec : nullptr, hat_rows, E);
   DMOE_STAMP(25);
   mask_topk_warps(k, B, size, order, prob, out);
   __syncthreads();
@@ -577,6 +581,7 @@ __device__ inline void block_route_steps(int E, int kb, int k, int B, float top_
 
 // Algorithm 1 for block b with the block's rows in global memory ([T, E] row-major). The
 // hat rows hold TopKMask(s_i, kb); every token keeps its k <= kb best coreset members.
+template <bool kTopK>
 __device__ inline void block_route_cta(int b, const float* probs, const float* probs_hat, int E,
                                        int kb, int k, int B, float top_p,
                                        int32_t* __restrict__ topk_idx,
@@ -585,7 +590,7 @@ __device__ inline void block_route_cta(int b, const float* probs, const float* p
                                        int32_t* __restrict__ coreset_size,
                                        uint32_t* __restrict__ spec = nullptr) {
   const size_t r0 = (size_t)b * B;
-  block_route_steps(
+  block_route_steps<kTopK>(
       E, kb, k, B, top_p,
       [&](int i, int e) { return probs_hat[(r0 + i) * E + e]; },
       [&](int i, int e) { return probs[(r0 + i) * E + e]; },
