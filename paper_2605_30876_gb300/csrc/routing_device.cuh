@@ -237,7 +237,7 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
   // nonzero entries, ids ascending: order key in the high word, the id's complement in the low
   // one (a larger number comes first); read two at a time
   __shared__ __align__(16) uint64_t nz_kid[kMaxExperts];
-  __shared__ int wcnt[2][8];
+  __shared__ int wcnt[8];
   __shared__ int s_size;
   __shared__ float fscr[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -362,12 +362,12 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     const bool zero = live && !in;
     const uint32_t bin = __ballot_sync(0xffffffffu, in), bzr = __ballot_sync(0xffffffffu, zero);
     const uint32_t bpos = __ballot_sync(0xffffffffu, live && st > 0.f);
-    if (lane == 0) wcnt[0][warp] = __popc(bin) | __popc(bzr) << 10 | __popc(bpos) << 20;
+    if (lane == 0) wcnt[warp] = __popc(bin) | __popc(bzr) << 10 | __popc(bpos) << 20;
     __syncthreads();
     int ahead = 0, all = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      ahead += w < warp ? wcnt[0][w] : 0;
-      all += wcnt[0][w];
+      ahead += w < warp ? wcnt[w] : 0;
+      all += wcnt[w];
     }
     const uint32_t below = (1u << lane) - 1u;
     const int n = all & 0x3ff, nnz = all >> 20;
@@ -426,58 +426,32 @@ __device__ inline int block_coreset_steps(int E, int k, int B, float top_p, HatF
     __syncthreads();   // st_s and order are rewritten by a later block of the same CTA
     return size;
   }
-  // p >= 1: every nonzero entry is in; sort them by ranks in parallel.
-  // compact the nonzero entries (and count the zero ones), in id order
+  // p >= 1: every nonzero entry is in, sorted by its rank; the zero entries follow by id.
   const bool nz = live && st > 0.f;
-  const bool z = live && !nz;
-  const uint32_t bnz = __ballot_sync(0xffffffffu, nz), bz = __ballot_sync(0xffffffffu, z);
+  const uint32_t bnz = __ballot_sync(0xffffffffu, nz);
   __syncthreads();   // wcnt and the lists are rewritten by a later block of the same CTA
-  if (lane == 0) {
-    wcnt[0][warp] = __popc(bnz);
-    wcnt[1][warp] = __popc(bz);
-  }
+  if (lane == 0) wcnt[warp] = __popc(bnz);
   __syncthreads();
-  int pnz = __popc(bnz & ((1u << lane) - 1u)), pz = __popc(bz & ((1u << lane) - 1u)), nnz = 0, nzero = 0;
+  int before = __popc(bnz & ((1u << lane) - 1u)), nnz = 0;   // nonzero entries with a lower id
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-    if (w < warp) {
-      pnz += wcnt[0][w];
-      pz += wcnt[1][w];
-    }
-    nnz += wcnt[0][w];
-    nzero += wcnt[1][w];
+    before += w < warp ? wcnt[w] : 0;
+    nnz += wcnt[w];
   }
-  if (nz) nz_kid[pnz] = (uint64_t)order_key(st) << 32 | (uint32_t)~tid;
+  const uint64_t me = (uint64_t)order_key(st) << 32 | (uint32_t)~tid;
+  if (nz) nz_kid[before] = me;
   __syncthreads();
   DMOE_STAMP(20);
-  // ranks of the nonzero entries -> sorted positions; zero entries after them by id
   if (nz) {
-    const uint64_t me = (uint64_t)order_key(st) << 32 | (uint32_t)~tid;
     int r = 0;
 #pragma unroll 8
     for (int j = 0; j < nnz; ++j) r += nz_kid[j] > me ? 1 : 0;
     order[r] = tid;
-    st_s[r] = st;
+  } else if (live) {
+    order[nnz + tid - before] = tid;
   }
-  if (z) order[nnz + pz] = tid;
   __syncthreads();
   DMOE_STAMP(21);
-  if (tid == 0) {
-    int m = nnz;
-    if (top_p < 1.f) {
-      float cum = 0.f;
-      for (int r = 0; r < nnz; ++r) {
-        cum += st_s[r];
-        if (cum >= top_p) {
-          m = r + 1;
-          break;
-        }
-      }
-    }
-    s_size = max(m, k);
-  }
-  __syncthreads();
-  const int size = s_size;
-  (void)nzero;
+  const int size = max(nnz, k);
   if (coreset != nullptr && live) coreset[tid] = (tid < size) ? order[tid] : -1;
   if (coreset_size != nullptr && tid == 0) coreset_size[0] = size;
   return size;
