@@ -95,7 +95,8 @@ struct GemmParams {
   // writes the dispatch's outputs n_unique, unique_ids and pos (the row of every (token,
   // slot), from topk_idx).
   const uint32_t* spec_words;
-  int n_blocks, blk;
+  int n_blocks, blk;      // (a block of 256 rows counts as two, which share its coreset:
+  int halves;             // halves = 1)
   const int32_t* topk_idx;
   int32_t* pos_out;
   int32_t* n_unique_out;
@@ -275,7 +276,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
       // Block top-k: poll every block's published coreset words until all are nonzero (a
       // nonzero word is complete), recording each block's members and, per expert, the
       // blocks that use it
-      const int nw = spec_words(p.k), total = p.n_blocks * nw;
+      const int nw = spec_words(p.k), total = (p.n_blocks >> p.halves) * nw;
       for (int i = lane; i < 2 * kMaxExperts; i += 32) s_bmask[i] = 0u;
       __syncwarp();
       bool bad = false;
@@ -288,7 +289,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
             all = false;
             continue;
           }
-          const int b = i / nw, r0 = 3 * (i % nw);
+          const int b = (i / nw) << p.halves, r0 = 3 * (i % nw);
 #pragma unroll
           for (int j = 0; j < 3; ++j) {
             if (r0 + j >= p.k) break;
@@ -296,7 +297,7 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
             if (e >= p.E) {
               bad = true;
             } else {
-              atomicOr(&s_bmask[2 * e + (b >> 5)], 1u << (b & 31));
+              atomicOr(&s_bmask[2 * e + (b >> 5)], (1u | (uint32_t)p.halves << 1) << (b & 31));
             }
           }
         }
@@ -1228,11 +1229,12 @@ int experts_ready_counters(int T, int E, int n_max) {
 }
 
 bool experts_spec_ok(const dmoe_layer_desc& d, int n_max) {
-  // blocks that fill a CTA's half of a token tile whole (expert_tile_unit), at most kSpecBlocks
-  // of them (a 64-bit block mask per expert)
-  return d.mode == DMOE_ROUTE_BLOCK && d.top_p <= 0.f && mask_top_k(d) == d.top_k &&
-         d.n_blocks >= 1 && d.n_blocks <= kSpecBlocks && expert_tile_unit(d.block_size) > 0 &&
-         n_max % expert_tile_unit(d.block_size) == 0 && d.n_experts <= kMaxExperts;
+  // blocks (or their halves) that fill a CTA's half of a token tile whole (expert_tile_unit), at
+  // most kSpecBlocks of them (a 64-bit block mask per expert)
+  const int part = expert_tile_part(d.block_size);
+  return d.mode == DMOE_ROUTE_BLOCK && d.top_p <= 0.f && mask_top_k(d) == d.top_k && part > 0 &&
+         d.n_blocks >= 1 && d.n_blocks * (d.block_size / part) <= kSpecBlocks &&
+         n_max % expert_tile_unit(part) == 0 && d.n_experts <= kMaxExperts;
 }
 
 cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
@@ -1279,8 +1281,9 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   gp.has_shared = has_shared ? 1 : 0;
   if (spec) {
     gp.spec_words = a.spec_words;
-    gp.n_blocks = a.spec_blocks;
-    gp.blk = a.T / a.spec_blocks;
+    gp.blk = expert_tile_part(a.T / a.spec_blocks);
+    gp.n_blocks = a.T / gp.blk;
+    gp.halves = gp.n_blocks > a.spec_blocks ? 1 : 0;
     gp.unit = expert_tile_unit(gp.blk);   // whole blocks
     gp.topk_idx = a.topk_idx;
     gp.pos_out = a.pos_out;

@@ -21,6 +21,7 @@ CASES = {
     "blocks_40x4_d384": SMALL.with_(block_size=40, n_blocks=4, d_model=384),
     "blocks_8x33": SMALL.with_(block_size=8, n_blocks=33, n_experts=8),
     "blocks_128x3": SMALL.with_(block_size=128, n_blocks=3),
+    "blocks_256x3": SMALL.with_(block_size=256, n_blocks=3),   # two halves, a CTA's each
     "blocks_48x9_d640": SMALL.with_(block_size=48, n_blocks=9, d_model=640, n_experts=16),
     # no half tile of whole blocks: the copied rows
     "blocks_72x3": SMALL.with_(block_size=72, n_blocks=3),
