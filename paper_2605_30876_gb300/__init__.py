@@ -161,8 +161,10 @@ def dmoe_workspace_size(desc: LayerDesc) -> int:
 
 
 def alloc_workspace(desc: LayerDesc, device="cuda") -> torch.Tensor:
-    """A zeroed uint8 device buffer of dmoe_workspace_size(desc) bytes (torch allocates)."""
+    """A zeroed uint8 buffer of dmoe_workspace_size(desc) bytes on `device` (torch allocates)."""
     ws = torch.empty(dmoe_workspace_size(desc), dtype=torch.uint8, device=device)
+    if not ws.is_cuda:   # a host image of a workspace: nothing was prepared at its address
+        return ws.zero_()
     dmoe_workspace_init(ws)
     return ws
 

@@ -51,6 +51,12 @@ def test_workspace_size_grows_with_tokens(dm):
     assert b < 64 * 2 ** 20
 
 
+def test_workspace_on_the_host(dm):
+    ws = dm.alloc_workspace(_desc(dm), device="cpu")
+    assert ws.device.type == "cpu" and ws.numel() == dm.dmoe_workspace_size(_desc(dm))
+    assert int(ws.count_nonzero()) == 0
+
+
 @pytest.mark.parametrize("kw,status", [
     (dict(top_k=0), 1), (dict(top_k=300), 1), (dict(n_experts=12), 2), (dict(n_experts=512), 2),
     (dict(top_k=17, n_experts=64), 2), (dict(d_model=200), 2), (dict(d_ff=100), 2),
