@@ -36,6 +36,7 @@
 // routing the gate/up phase streams weights at 6.5 TB/s (a copy: 6.7).
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "dmoe_internal.cuh"
@@ -1210,6 +1211,36 @@ int max_smem_optin() {
   return v;
 }
 
+// The pairs of CTAs of the expert launch that the current device runs at once; on the first call per
+// device it also raises the kernels' limit of dynamic shared memory to `smem`, which is set per
+// device.
+cudaError_t resident_pairs(int smem, int* pairs) {
+  static std::atomic<int> known[32];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  *pairs = dev < 32 ? known[dev].load(std::memory_order_acquire) : 0;
+  if (*pairs > 0) return cudaSuccess;
+  for (auto* kernel : {moe_experts_kernel<false, false>, moe_experts_kernel<true, false>,
+                       moe_experts_kernel<false, true>, moe_experts_kernel<true, true>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kCluster;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCluster);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveClusters(pairs, moe_experts_kernel<false, false>, &cfg);
+  if (e == cudaSuccess && dev < 32) known[dev].store(*pairs, std::memory_order_release);
+  return e;
+}
+
 }  // namespace
 
 #ifdef DMOE_TRACE
@@ -1341,27 +1372,19 @@ cudaError_t launch_experts(const ExpertArgs& a, cudaStream_t s) {
   if (gp.n_acc > 4) gp.n_acc = 4;
   gp.tmem_cols = (uint32_t)gp.n_acc * gp.acc_cols;
   const size_t smem = fixed + (size_t)gp.a_stages * kATileBytes + gp.b_stages * row_slot;
-  static int attr_dev_mask = 0;  // the dynamic smem limit is a per-device function attribute
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev >= 31 || !(attr_dev_mask & (1 << dev))) {
-    cudaError_t e = cudaSuccess;
-    for (auto* kernel : {moe_experts_kernel<false, false>, moe_experts_kernel<true, false>,
-                         moe_experts_kernel<false, true>, moe_experts_kernel<true, true>})
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
-    if (e != cudaSuccess) return e;
-    if (dev < 31) attr_dev_mask |= 1 << dev;
-  }
-  int grid = device_sm_count() / kCluster * kCluster;
+  int pairs_max = 0;
+  cudaError_t e = resident_pairs(limit, &pairs_max);
+  if (e != cudaSuccess) return e;
+  // (every pair owns its first unit, which other pairs' down units may wait for: no more pairs than
+  // can run at once)
+  int grid = std::min(device_sm_count() / kCluster, pairs_max) * kCluster;
   if (grid > kMaxPersistentCtas) grid = kMaxPersistentCtas;
   if (grid < kCluster) return cudaErrorInvalidConfiguration;
   prof_begin(DMOE_KERNEL_EXPERTS, s);
-  cudaError_t e = launch_cluster(far ? (spec ? moe_experts_kernel<true, true> : moe_experts_kernel<false, true>)
-                                     : (spec ? moe_experts_kernel<true, false>
-                                             : moe_experts_kernel<false, false>),
-                                 dim3(grid), dim3(kThreads), smem, s, kCluster,
-                                 !prof_serial(DMOE_KERNEL_EXPERTS), m, gp);
+  e = launch_cluster(
+      far ? (spec ? moe_experts_kernel<true, true> : moe_experts_kernel<false, true>)
+          : (spec ? moe_experts_kernel<true, false> : moe_experts_kernel<false, false>),
+      dim3(grid), dim3(kThreads), smem, s, kCluster, !prof_serial(DMOE_KERNEL_EXPERTS), m, gp);
   prof_end(DMOE_KERNEL_EXPERTS, s);
   if (e != cudaSuccess) return e;
 
