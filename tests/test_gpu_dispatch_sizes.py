@@ -39,4 +39,6 @@ def test_dispatch_records_bad_ids(T, fault, code):
     idx[T - 1, 1] = 16 if fault == "id" else idx[T - 1, 0]
     _, ws = P.gpu_dispatch(shape, torch.from_numpy(idx).cuda())
     st, info = P.dm().dmoe_get_device_error(ws)
-    assert st == 5 and info[0] in (code, 4)   # 4: the pairs do not add up, if recorded first
+    # 4 (the pairs do not add up) can be recorded first only where the one launch both counts and
+    # checks, and only for the bad id: a doubled expert's pairs are all counted there
+    assert st == 5 and info[0] in ((code, 4) if T == 512 and fault == "id" else (code,))

@@ -1,9 +1,11 @@
 """The expert launches where their tiles can go wrong, against the CPU oracle. The general one (more
 than 64 tokens): tiles of 32 to 256 token rows with remainders, blocks that fill half tiles in twos or
 fours, blocks that fill none, d and I of an odd number of 128-row tiles, more token tiles than
-one, fewer units than clusters, and gate and up weights that no single copy can bring. The
-decode-size one: both unit heights, the smallest and the largest token count, outputs kept by
-few tokens, and the same two forms of the weights' copies."""
+one, and fewer units than clusters. The decode-size one: both unit heights, the smallest and the
+largest token count, and outputs kept by few tokens. Both with every form of the gate and up
+weights' copies: one copy for both tensors, the gate's or the up's address the lower one, in the
+routed experts and the shared one apart; and a copy for each, which any pair that is one tensor
+(distance 0 is no stride) brings about for the other pair too."""
 import numpy as np
 import pytest
 import torch
@@ -45,15 +47,26 @@ CASES = {
 }
 
 
-@pytest.mark.parametrize("one_tensor", [False, True])
+# (routed, shared): 0: the up tensor is the gate tensor; 1: gate at the lower address; 2: up there
+FORMS = {"gate_first": (1, 1), "up_first": (2, 2), "shared_up_first": (1, 2), "one_tensor": (0, 0),
+         "routed_apart": (1, 0), "routed_apart_up_first": (2, 0), "shared_apart": (0, 1)}
+
+
+@pytest.mark.parametrize("form", FORMS)
 @pytest.mark.parametrize("name", CASES)
-def test_layer_matches_oracle(name, one_tensor):
+def test_layer_matches_oracle(name, form):
     shape = CASES[name]
     m = P.dm()
     dev, host = P.make(shape, seed=7)
-    if one_tensor:   # W_up is W_gate: at distance 0 the two are not one strided tensor
-        for a, b in (("w_up", "w_gate"), ("ws_up", "ws_gate")):
-            dev[a], host[a] = dev[b], host[b]
+    for prefix, how in zip(("w", "ws"), FORMS[form]):
+        gate, up = f"{prefix}_gate", f"{prefix}_up"
+        if dev[gate] is None:
+            continue
+        if how == 0:
+            dev[up], host[up] = dev[gate], host[gate]
+            continue
+        both = torch.stack([dev[gate], dev[up]] if how == 1 else [dev[up], dev[gate]])
+        dev[gate], dev[up] = both[how - 1], both[2 - how]
     from paper_2605_30876_gb300.layer import MoELayer
     layer = MoELayer.from_shape(shape, dev)
     y = layer.forward(dev["x"]).clone()
