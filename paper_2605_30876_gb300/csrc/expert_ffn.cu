@@ -174,8 +174,9 @@ __device__ uint64_t g_trace[kMaxPersistentCtas * 64];
 // top-k form (GemmParams::spec_words), compiled separately so that the other form carries none
 // of its code. kFar: W_gate and W_up too far apart for one map (2^40 bytes or more: allocations
 // in two address ranges; or the same tensor), 16 rows of each over K = 128 in a box of their own,
-// filling two slots. 256 tokens, token routing, 128 experts of I = 384: 110 us with one map, 125
-// so, 137 with 16 rows over K = 64 a box (2 KB copies are below the HBM rate).
+// filling two slots, issued by eight lanes. Token routing, 128 experts of I = 384, 256 / 128 / 2048
+// tokens: 112.5 / 106.3 / 182.8 us with one map, 118.9 / 112.7 / 187.3 so, 125.1 / 119.0 / 190.5
+// with all boxes from one lane; 16 rows over K = 64 a box are slower still (2 KB copies).
 template <bool kSpec, bool kFar>
 __global__ void __launch_bounds__(kThreads, 1)
 moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
