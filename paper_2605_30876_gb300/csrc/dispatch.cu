@@ -12,7 +12,7 @@
 // the counts are cheap enough to be made in every CTA.
 // Every sum is of integers, and each expert's rows are ordered by token, the canonical
 // dispatch form. An id outside [0, E) or an expert twice in one token is recorded as a fault;
-// the outputs are then unspecified (rows stay in range).
+// the outputs are then unspecified: every pos is in range, some entries of rows are not written.
 #include "block_reduce.cuh"
 #include "dmoe_internal.cuh"
 #include "trace_log.cuh"
@@ -187,6 +187,9 @@ dispatch_place_kernel(const int32_t* __restrict__ topk_idx, int T, int E, int k,
         r = -1;
       }
     }
+    // (a bad id has no row; its place is one that the combine can read. Checked there instead, it
+    // took the combine of 2048 tokens 2 us longer)
+    if (r < 0 && p < p1) pos[t0 * k + p] = 0;
     if (xperm != nullptr && p < p1) {
       s_r[p - p0] = r;
       s_t[p - p0] = t0 + p / k;

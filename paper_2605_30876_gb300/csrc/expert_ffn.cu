@@ -987,7 +987,9 @@ moe_experts_kernel(const __grid_constant__ Maps tm, const GemmParams p) {
   }
 }
 
-// xperm[r, :] = x[rows[r] / k, :]; block 0 also clears the gate/up tile counters.
+// xperm[r, :] = x[rows[r] / k, :]; block 0 also clears the gate/up tile counters. After a fault that
+// the dispatch recorded (a bad id, an expert twice in a token) entries of `rows` are whatever the
+// caller's buffer held: they are kept in range.
 __global__ void __launch_bounds__(256)
 gather_kernel(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ rows,
               __nv_bfloat16* __restrict__ xperm, int32_t* __restrict__ h_ready, int n_ready,
@@ -999,7 +1001,7 @@ gather_kernel(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ r
     for (int i = threadIdx.x; i < n_ready; i += blockDim.x) h_ready[i] = 0;
   const int vec = d / 8;  // uint4 per row
   for (int r = blockIdx.x; r < pairs; r += gridDim.x) {
-    const int t = rows[r] / k;
+    const int t = (int)min((uint32_t)rows[r], (uint32_t)pairs - 1u) / k;
     const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)t * d);
     uint4* dst = reinterpret_cast<uint4*>(xperm + (size_t)r * d);
     for (int i = threadIdx.x; i < vec; i += blockDim.x) dst[i] = src[i];
