@@ -30,11 +30,19 @@ SHAPES = {
 }
 
 
-@pytest.mark.parametrize("shape", SHAPES.values(), ids=SHAPES)
-def test_bounded_wait_times_out_and_the_workspace_recovers(shape):
+# the shared expert's two tensors are one, which makes every gate/up pair come in boxes of its own
+APART = {"block_apart": TINY.with_(d_ff_shared=128), "general_block_apart": GENERAL,
+         "general_token_apart": GENERAL.with_(mode=ROUTE_TOKEN)}
+
+
+@pytest.mark.parametrize("name", [*SHAPES, *APART])
+def test_bounded_wait_times_out_and_the_workspace_recovers(name):
     m = P.dm()
     from paper_2605_30876_gb300.layer import MoELayer
+    shape = {**SHAPES, **APART}[name]
     dev, host = P.make(shape, seed=3)
+    if name in APART:
+        dev["ws_up"], host["ws_up"] = dev["ws_gate"], host["ws_gate"]
     layer = MoELayer.from_shape(shape, dev)
     layer.forward(dev["x"])
     assert m.dmoe_get_device_error(layer.ws)[0] == 0
